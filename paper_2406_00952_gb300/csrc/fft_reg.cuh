@@ -37,6 +37,44 @@ template <typename R> __device__ __forceinline__ cx<R> w96(int k);
 template <> __device__ __forceinline__ float2 w96<float>(int k) { return c_w96f[k]; }
 template <> __device__ __forceinline__ double2 w96<double>(int k) { return c_w96d[k]; }
 
+// The same roots with a compile-time index (the unrolled register DFTs): cos(2 pi k / 96), k = 0 .. 24,
+// rounded to FP64, and the octant symmetries.  They fold into the instructions, so a unit that uses the
+// register DFTs alone needs no table upload.
+__device__ __forceinline__ constexpr double cos96(int k) {
+  constexpr double c[25] = {
+    1.0, 0.9978589232386035, 0.9914448613738104, 0.9807852804032304,
+    0.9659258262890683, 0.9469301294951057, 0.9238795325112867, 0.8968727415326883,
+    0.8660254037844386, 0.8314696123025452, 0.7933533402912352, 0.7518398074789774,
+    0.7071067811865476, 0.6593458151000688, 0.6087614290087207, 0.5555702330196022,
+    0.5, 0.4422886902190013, 0.3826834323650898, 0.3214394653031616,
+    0.25881904510252074, 0.19509032201612828, 0.1305261922200516, 0.06540312923014306,
+    0.0};
+  return k <= 24 ? c[k] : k <= 48 ? -c[48 - k] : k <= 72 ? -c[k - 48] : c[96 - k];
+}
+template <typename R> __device__ __forceinline__ constexpr cx<R> root96(int k) {   // exp(-2 pi i k / 96)
+  cx<R> w{};
+  w.x = (R)cos96(k);
+  w.y = (R)(k <= 72 ? -cos96((k + 72) % 96) : -cos96(k - 24));
+  return w;
+}
+
+// exp(-2 pi i k / 64), 0 <= k < 32, with a compile-time index (the zeta = pi twist of the time lines)
+__device__ __forceinline__ constexpr double cos64(int k) {
+  constexpr double c[17] = {
+    1.0, 0.9951847266721969, 0.9807852804032304, 0.9569403357322088,
+    0.9238795325112867, 0.881921264348355, 0.8314696123025452, 0.773010453362737,
+    0.7071067811865476, 0.6343932841636455, 0.5555702330196022, 0.47139673682599764,
+    0.3826834323650898, 0.2902846772544624, 0.19509032201612828, 0.0980171403295606,
+    0.0};
+  return k <= 16 ? c[k] : -c[32 - k];
+}
+template <typename R> __device__ __forceinline__ constexpr cx<R> root64(int k) {
+  cx<R> w{};
+  w.x = (R)cos64(k);
+  w.y = (R)-(k <= 16 ? cos64(16 - k) : cos64(k - 16));
+  return w;
+}
+
 template <typename T>
 __device__ __forceinline__ void r2(T& a, T& b) { T t = cadd(a, b); b = csub(a, b); a = t; }
 
@@ -113,9 +151,14 @@ __device__ __forceinline__ void reg_dft(T* x, bool inv) {
     for (int k1 = 0; k1 < A; ++k1) {
       T v = t[k1];
       if (b * k1) {
-        T w = w96<R>((b * k1 * (96 / Q)) % 96);
-        if (inv) w.y = -w.y;
-        v = cmul(v, w);
+        const int k = (b * k1 * (96 / Q)) % 96;
+        if (k == 24) {                       // a quarter turn is exact
+          v = inv ? cmul_pi(v) : cmul_mi(v);
+        } else {
+          T w = root96<R>(k);
+          if (inv) w.y = -w.y;
+          v = cmul(v, w);
+        }
       }
       x[b + B * k1] = v;
     }

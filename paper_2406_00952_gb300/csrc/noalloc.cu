@@ -25,6 +25,7 @@ namespace pcb {
 struct TableLayout { size_t kap, mud, muf, twdd, twdf, twtd, twtf, pred, pref, ax, ay, dg, ms, bytes; };
 int validate_desc(const pcb_desc* d);
 void init_geom(const pcb_desc* d, Geom& g);
+void reshape_geom(Geom& g);
 size_t table_layout(const Geom& g, TableLayout& t);
 void fill_tables(const pcb_desc* d, const Geom& g, const TableLayout& t, unsigned char* host);
 void bind_tables(Geom& g, const TableLayout& t, unsigned char* tb);
@@ -78,6 +79,8 @@ extern "C" int pcb_precond_apply_noalloc(const pcb_desc* desc, int kind, int pre
   Geom g;
   init_geom(desc, g);
   // the arena holds one FP32 scratch buffer of 2mn values: unpadded layout, kernels of precond.cu
+  g.tune = TUNE_NO_LANE;
+  reshape_geom(g);
   g.lr = g.N;
   g.mp = g.m;
   g.time_blocks[1] = (g.m + g.time_cpb[1] - 1) / g.time_cpb[1];

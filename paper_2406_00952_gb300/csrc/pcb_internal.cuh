@@ -136,6 +136,11 @@ struct Geom {
   int dst_blocks_i[2], dst_blocks_j[2]; // blocks of the x1-line and x2-line DST passes
   int time_cpb[2];                // spatial columns per block of the time pass
   int time_blocks[2];
+  // one-line-per-lane passes (precond_lane.cuh), index 0 = FP64 apply, 1 = FP32 apply: codes of the
+  // spatial and the time kernels (lane_space_code, lane_time_code; 0: this instance takes the kernels
+  // of precond.cu / precond_pipe.cu in that precision) and their block counts
+  int lane_sp[2], lane_tm[2];
+  int ls_blocks[2], lt_blocks[2];
   int tune;                       // kernel choices of the autotuner (TUNE_* bits; 0 = defaults)
   int mv_tchunk;                  // time steps per thread in the theta = 1 matvec
   int mv_blocks;                  // blocks of the matvec
@@ -151,7 +156,7 @@ struct Geom {
   const float2* twd_f;
   const double2* twt_d;           // n: exp(-2 pi i k / n)
   const float2* twt_f;
-  const double2* pre_d;           // n: exp(-i pi t / n)   (zeta = pi scaling, D_omega conj)
+  const double2* pre_d;           // 2n: exp(-i zeta t / n) (D_omega conj; the zeta = pi kernels read all 2n)
   const float2* pre_f;
   const double* axs;              // var_a: tau/h^2 * ax  (N x (N+1))
   const double* ays;              //        tau/h^2 * ay  ((N+1) x N)
@@ -163,7 +168,7 @@ struct Geom {
 // Autotuner choices (Geom::tune): kernel families the FP32 apply may not use, and the tile-size
 // scale of the tile kernels (bits 4-5: 0 = default, 1 = half, 2 = double the per-tile element budget)
 enum { TUNE_NO_PIPE_DST = 1, TUNE_NO_PIPE_TIME = 2, TUNE_NO_HANDOFF = 4, TUNE_TIME512_3BLK = 8,
-       TUNE_TIME512_4BLK = 64 };
+       TUNE_TIME512_4BLK = 64, TUNE_NO_LANE = 128 };
 __host__ __device__ inline int tune_budget_shift(int tune) { return (tune >> 4) & 3; }
 
 // per-instance Krylov scalars (MINRES and GMRES share the struct)
@@ -236,6 +241,20 @@ __host__ __device__ inline int fam_code(int index) {
   return (1 << index) | tm | ev;
 }
 
+// codes of the one-line-per-lane kernels: spatial lines of M = 2L points, 1 + index of M (+ 11 for the
+// DCT-I); time lines of n = 2^k, k (+ 10 for general zeta).  0: no such kernel.
+constexpr int kLaneLengths[11] = {32, 48, 64, 96, 128, 192, 256, 384, 512, 768, 1024};
+inline int lane_space_code(int M, bool ev) {
+  for (int k = 0; k < 11; ++k)
+    if (kLaneLengths[k] == M) return 1 + k + (ev ? 11 : 0);
+  return 0;
+}
+inline int lane_time_code(int n, bool gz) {
+  for (int k = 1; k <= 10; ++k)
+    if (n == 1 << k) return k + (gz ? 10 : 0);
+  return 0;
+}
+
 // ------------------------------------------------------------------------------------------
 // host-side launch helpers (defined in runtime.cu)
 // ------------------------------------------------------------------------------------------
@@ -250,6 +269,8 @@ struct Batch {
   const int* off_dst_i[2]; int tot_dst_i[2];
   const int* off_dst_j[2]; int tot_dst_j[2];
   const int* off_time[2];  int tot_time[2];
+  const int* off_ls[2];    int tot_ls[2];      // one-line-per-lane spatial and time passes
+  const int* off_lt[2];    int tot_lt[2];
   const int* off_mv;    int tot_mv;
   const int* off_vec;   int tot_vec;
   double* partial;        // reduction partials
@@ -264,6 +285,11 @@ struct Batch {
   const int* fam_dst;
   const int* fam_time;
   int fam_dst_set, fam_time_set;
+  // one-line-per-lane kernels: device arrays [count] of Geom::lane_sp / lane_tm per precision, and the
+  // codes present (bit `code`) among the instances with work
+  const int* lane_sp[2];
+  const int* lane_tm[2];
+  unsigned lane_sp_set[2], lane_tm_set[2];
   int t512v;              // 1 / 2: the n = 512 time pass runs its three / four-blocks-per-SM variant
                           // (every instance of the batch that takes that pass chose it)
   int fem_m;              // > 0: a single finite-element instance with m = fem_m spatial points
@@ -273,5 +299,8 @@ struct Batch {
   Sel sel() const { Sel s; s.active = active; s.fam = filt; s.want = filt_want; return s; }
   size_t dst_smem[2], time_smem[2];   // dynamic shared memory per block, per precision
 };
+
+// device ints fill_batch needs for `count` instances: 12 offset arrays of count + 1, 6 code arrays of count
+inline size_t batch_ints(int count) { return (size_t)12 * (count + 1) + (size_t)6 * count; }
 
 }  // namespace pcb

@@ -740,9 +740,58 @@ static cudaError_t time_pass(const Batch& B, int kind) {
   return cudaSuccess;
 }
 
+cudaError_t lane_rows_f32(const Batch& B, Sel sel, int M, bool ev, int stage, int in_sel, int out_sel);
+cudaError_t lane_rows_f64(const Batch& B, Sel sel, int M, bool ev, int stage, int in_sel, int out_sel);
+cudaError_t lane_cols_f32(const Batch& B, Sel sel, int M, bool ev, int stage, int in_sel, int out_sel);
+cudaError_t lane_cols_f64(const Batch& B, Sel sel, int M, bool ev, int stage, int in_sel, int out_sel);
+cudaError_t lane_time_f32(const Batch& B, Sel sel, int n, bool gz, int kind, int in_sel, int out_sel);
+cudaError_t lane_time_f64(const Batch& B, Sel sel, int n, bool gz, int kind, int in_sel, int out_sel);
+
+// The five passes with one line per lane (precond_lane.cuh), for the instances whose codes say so:
+//   1: along x2, input -> scratch;  2: along x1, transposed;  3: time;  4: along x1 (now the row
+//   index), in place;  5: along x2, transposed back, to the output.
+// FP32 works in the two padded scratch buffers (-1, -2).  FP64 has one scratch buffer: pass 2 parks its
+// transposed result in the output vector, which pass 3 reads back (the input is no longer needed then,
+// so input and output may be the same vector).  A launch per kernel family present, over the
+// instances of that family.
+template <typename R>
+static cudaError_t lane_passes(const Batch& B, int kind, int in_slot, int out_slot) {
+  constexpr int p = sizeof(R) == 4;
+  const int first = -1, second = p ? -2 : out_slot, timed = p ? -2 : -1;
+  auto spatial = [&](int stage, int in_sel, int out_sel) {
+    const unsigned set = B.lane_sp_set[p];
+    for (int code = 1; code <= 22; ++code) {
+      if (!(set >> code & 1)) continue;
+      Sel s{B.active, set == 1u << code && B.tot_dst_i[p] == 0 ? nullptr : B.lane_sp[p], code};
+      const int M = kLaneLengths[(code - 1) % 11];
+      const bool ev = code > 11, rows = stage == 1 || stage == 4;
+      const cudaError_t e = p ? (rows ? lane_rows_f32 : lane_cols_f32)(B, s, M, ev, stage, in_sel, out_sel)
+                              : (rows ? lane_rows_f64 : lane_cols_f64)(B, s, M, ev, stage, in_sel, out_sel);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  };
+  cudaError_t e;
+  if ((e = spatial(1, in_slot, first)) != cudaSuccess) return e;
+  if ((e = spatial(2, first, second)) != cudaSuccess) return e;
+  const unsigned set = B.lane_tm_set[p];
+  for (int code = 1; code <= 20; ++code) {
+    if (!(set >> code & 1)) continue;
+    Sel s{B.active, set == 1u << code && B.tot_dst_i[p] == 0 ? nullptr : B.lane_tm[p], code};
+    const int n = 1 << ((code - 1) % 10 + 1);
+    if ((e = (p ? lane_time_f32 : lane_time_f64)(B, s, n, code > 10, kind, second, timed)) != cudaSuccess) return e;
+  }
+  if ((e = spatial(4, timed, timed)) != cudaSuccess) return e;
+  return spatial(5, timed, out_slot);
+}
+
 template <typename R>
 static cudaError_t precond_passes(const Batch& B, int kind, int in_slot, int out_slot) {
   cudaError_t e;
+  if (B.lane_sp_set[sizeof(R) == 4]) {
+    if ((e = lane_passes<R>(B, kind, in_slot, out_slot)) != cudaSuccess) return e;
+    if (B.tot_dst_i[sizeof(R) == 4] == 0) return cudaSuccess;
+  }
   if ((e = dst_pass<R>(B, 1, in_slot, -1)) != cudaSuccess) return e;
   if ((e = dst_pass<R>(B, 2, -1, -1)) != cudaSuccess) return e;
   if ((e = time_pass<R>(B, kind)) != cudaSuccess) return e;

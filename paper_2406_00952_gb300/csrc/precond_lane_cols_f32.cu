@@ -1,0 +1,22 @@
+// FP32 spatial passes along the rows of a slice with a transposed result (precond_lane.cuh): pass 2 stays
+// in the FP32 scratch, pass 5 writes the FP64 output.
+#include "precond_lane.cuh"
+
+namespace pcb {
+namespace {
+template <int M, bool EV>
+struct Cols {
+  static cudaError_t run(const Batch& B, Sel sel, int stage, int in_sel, int out_sel) {
+    return stage == 2 ? lane::cols_pass<float, M, EV, false>(B, sel, in_sel, out_sel, 0)
+                      : lane::cols_pass<float, M, EV, true>(B, sel, in_sel, out_sel, 1);
+  }
+};
+
+}  // namespace
+
+cudaError_t lane_cols_f32(const Batch& B, Sel sel, int M, bool ev, int stage, int in_sel, int out_sel) {
+  return ev ? lane::by_length<true, Cols>(M, B, sel, stage, in_sel, out_sel)
+            : lane::by_length<false, Cols>(M, B, sel, stage, in_sel, out_sel);
+}
+
+}  // namespace pcb

@@ -23,6 +23,7 @@
 // instance takes these kernels for all of its DST passes or for none; see pipe_dst_p.
 #include <algorithm>
 
+#include "f32_convert.cuh"
 #include "fft_reg.cuh"
 
 namespace pcb {
@@ -53,57 +54,6 @@ __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {   // a * conj(b)
   c.x = a.x * b.x + a.y * b.y;
   c.y = a.y * b.x - a.x * b.y;
   return c;
-}
-
-// FP64 <-> FP32 conversions with integer operations.  The conversion instructions run on the FP64
-// pipe, which is narrow on this GPU and became the bottleneck of the passes that read or write
-// the FP64 vectors.  IEEE-754 binary64 -> binary32, round to nearest even: for results in the
-// normal FP32 range the rounded value is the top 31 bits of (exponent - 896, mantissa >> 29)
-// plus one when the dropped 29 bits exceed half, or equal half and the kept value is odd (a
-// carry into the exponent gives the right next binade, or infinity).  Zeros keep their sign;
-// the rare remaining cases (FP32 subnormals, overflow, infinities, NaN) use the instruction.
-__device__ __forceinline__ float d2f(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned ah = hi & 0x7fffffffu, e = ah >> 20;
-  if (e - 897u <= 253u) {
-    const unsigned m = (ah << 3) | (lo >> 29);
-    const unsigned rem = lo & 0x1fffffffu;
-    const unsigned rnd = (unsigned)(rem > 0x10000000u) | ((unsigned)(rem == 0x10000000u) & m & 1u);
-    return __uint_as_float(((m - (896u << 23)) + rnd) | (hi & 0x80000000u));
-  }
-  if ((ah | lo) == 0u) return __uint_as_float(hi & 0x80000000u);
-  return __double2float_rn(x);
-}
-// binary32 -> binary64 (exact): exponent rebiased by 896, mantissa moved up by 29 bits
-__device__ __forceinline__ double f2d(float f) {
-  const unsigned b = __float_as_uint(f), e = (b >> 23) & 0xffu;
-  if (e - 1u < 254u) {
-    const unsigned hi = (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20));
-    return __hiloint2double((int)hi, (int)(b << 29));
-  }
-  if ((b & 0x7fffffffu) == 0u) return __hiloint2double((int)(b & 0x80000000u), 0);
-  return (double)f;
-}
-__device__ __forceinline__ float to_f32(float v) { return v; }
-__device__ __forceinline__ float to_f32(double v) { return d2f(v); }
-// The gather of pass 1 converts every kF2FEvery-th register of a line with the conversion
-// instruction and the rest with integer operations: both round to nearest even, and the mix
-// shares the work between the FP64 pipe and the integer pipe.
-constexpr int kF2FEvery = 2;
-__device__ __forceinline__ float to_f32_at(float v, int) { return v; }
-__device__ __forceinline__ float to_f32_at(double v, int q) {
-  return (kF2FEvery > 0 && q % kF2FEvery == kF2FEvery - 1) ? __double2float_rn(v) : d2f(v);
-}
-template <typename T> __device__ __forceinline__ T from_f32(float v);
-template <> __device__ __forceinline__ float from_f32<float>(float v) { return v; }
-template <> __device__ __forceinline__ double from_f32<double>(float v) { return f2d(v); }
-// pass 5's FP64 results: every kF2DEvery-th register through the conversion instruction
-constexpr int kF2DEvery = 2;
-template <typename T> __device__ __forceinline__ T from_f32_at(float v, int j) {
-  if constexpr (sizeof(T) == 8) {
-    if (kF2DEvery > 0 && j % kF2DEvery == kF2DEvery - 1) return (double)v;
-  }
-  return from_f32<T>(v);
 }
 
 // ------------------------------------------------------------------------------------------

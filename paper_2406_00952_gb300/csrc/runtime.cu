@@ -77,6 +77,9 @@ int pipe_dst_code(const Geom& g);
 int pipe_time_code(const Geom& g);
 int pipe_time_cols(int n, int zeta_pi);
 int pipe_dst_lines(int L);
+int lane_space_lines(int M, int p);
+int lane_time_columns(int n, bool gz, int p);
+int lane_time_tiles(int n);
 cudaError_t upload_constants();
 struct TableLayout { size_t kap, mud, muf, twdd, twdf, twtd, twtf, pred, pref, ax, ay, dg, ms, bytes; };
 cudaError_t mg_setup(Geom& g, void* ws, const double* a_edges_host, double a0);
@@ -122,7 +125,7 @@ struct pcb_problem {
   Slots hS;
   Slots* dS = nullptr;
   Scal* dSc = nullptr;
-  int* doff = nullptr;            // 12 offset arrays of length 2
+  int* doff = nullptr;            // offset and code arrays (batch_ints(1))
   double* partial = nullptr;
   Scal* hSc = nullptr;            // pinned host copy
   Slots* hSpin = nullptr;         // pinned staging for slot uploads
@@ -183,6 +186,30 @@ int vec_blocks_for(long long len) {
 
 int pow2_floor(int v) { int p = 1; while (p * 2 <= v) p *= 2; return p; }
 
+// The one-line-per-lane passes (precond_lane.cuh) take every instance of the transform route whose
+// spatial and time lines they cover, in FP32 and FP64; finite elements keep the passes of precond.cu,
+// whose per-mode step wants the vector layout.  FP64 time lines stop at 512 steps: a pair of 32-point
+// rows does not fit the registers.  Such an instance has no blocks in the other kernels' launches.
+void set_lane_shapes(Geom& g) {
+  for (int p = 0; p < 2; ++p) {
+    g.lane_sp[p] = g.lane_tm[p] = g.ls_blocks[p] = g.lt_blocks[p] = 0;
+    if (g.mg_route || g.fem || (g.tune & TUNE_NO_LANE) || (p == 0 && g.n > 512)) continue;
+    const int sp = lane_space_code(g.M, g.bc == PCB_BC_NEUMANN), tm = lane_time_code(g.n, !g.zeta_pi);
+    if (!sp || !tm) continue;
+    g.lane_sp[p] = sp;
+    g.lane_tm[p] = tm;
+    const int lines = lane_space_lines(g.M, p), cols = lane_time_columns(g.n, !g.zeta_pi, p);
+    g.ls_blocks[p] = g.n * ((g.N + lines - 1) / lines);
+    const int tiles = g.N * ((g.N + cols - 1) / cols), per = lane_time_tiles(g.n);
+    g.lt_blocks[p] = (tiles + per - 1) / per;
+    g.dst_blocks_i[p] = g.dst_blocks_j[p] = g.time_blocks[p] = 0;
+    if (p == 1) {        // the padded layout (two FP32 buffers) of the FP32 passes
+      g.lr = g.L + 16;
+      g.mp = (long long)g.N * g.lr;
+    }
+  }
+}
+
 void set_shapes(Geom& g) {
   const int pd = pipe_dst_p(g), pt = pipe_time_p(g);   // pipelined FP32 passes: 256/P lines a tile
   g.lr = pd ? g.L + 16 : g.N;      // + 16: rows stay 64-byte aligned, stride off a power of two
@@ -212,6 +239,7 @@ void set_shapes(Geom& g) {
     if (p == 1 && (pipe_time_code(g) & 64)) g.time_blocks[p] = g.N * ((g.N + cpb - 1) / cpb);   // rows of points
   }
   matvec_shape(g);
+  set_lane_shapes(g);
   g.vec_blocks = vec_blocks_for(2 * g.mn);
 }
 
@@ -263,6 +291,8 @@ static int build_offsets(const std::vector<Geom>& gs, std::vector<int>& host_off
       case 1: nb = g.dst_blocks_j[p]; break;
       case 2: nb = g.time_blocks[p]; break;
       case 3: nb = g.mv_blocks; break;
+      case 5: nb = g.ls_blocks[p]; break;
+      case 6: nb = g.lt_blocks[p]; break;
       default: nb = g.vec_blocks; break;
     }
     tot += nb;
@@ -272,22 +302,24 @@ static int build_offsets(const std::vector<Geom>& gs, std::vector<int>& host_off
   return 0;
 }
 
-// Fill B's offset tables for `gs` into the device int buffer `doff` (12 arrays of count+1).
+// Fill B's offset tables and kernel codes for `gs` into the device int buffer `doff` (batch_ints(count)).
 namespace pcb {
 int fill_batch(Batch& B, const std::vector<Geom>& gs, int* doff, cudaStream_t st, std::vector<int>& staging) {
   const int count = (int)gs.size();
   staging.clear();
-  int tots[8];
-  // order: dst_i[0], dst_i[1], dst_j[0], dst_j[1], time[0], time[1], mv, vec
-  const int which[8] = {0, 0, 1, 1, 2, 2, 3, 4};
-  const int prec[8] = {0, 1, 0, 1, 0, 1, 0, 0};
-  for (int a = 0; a < 8; ++a) build_offsets(gs, staging, tots[a], which[a], prec[a]);
+  int tots[12];
+  // order: dst_i[0], dst_i[1], dst_j[0], dst_j[1], time[0], time[1], mv, vec, ls[0], ls[1], lt[0], lt[1]
+  const int which[12] = {0, 0, 1, 1, 2, 2, 3, 4, 5, 5, 6, 6};
+  const int prec[12] = {0, 1, 0, 1, 0, 1, 0, 0, 0, 1, 0, 1};
+  for (int a = 0; a < 12; ++a) build_offsets(gs, staging, tots[a], which[a], prec[a]);
   CK(cudaMemcpyAsync(doff, staging.data(), staging.size() * sizeof(int), cudaMemcpyHostToDevice, st));
   const int stride = count + 1;
   for (int p = 0; p < 2; ++p) {
     B.off_dst_i[p] = doff + (0 + p) * stride; B.tot_dst_i[p] = tots[0 + p];
     B.off_dst_j[p] = doff + (2 + p) * stride; B.tot_dst_j[p] = tots[2 + p];
     B.off_time[p] = doff + (4 + p) * stride;  B.tot_time[p] = tots[4 + p];
+    B.off_ls[p] = doff + (8 + p) * stride; B.tot_ls[p] = tots[8 + p];
+    B.off_lt[p] = doff + (10 + p) * stride; B.tot_lt[p] = tots[10 + p];
     B.dst_smem[p] = 0; B.time_smem[p] = 0;
     for (const Geom& g : gs) {
       B.dst_smem[p] = std::max(B.dst_smem[p], dst_smem_bytes(g, p));
@@ -332,7 +364,19 @@ int fill_batch(Batch& B, const std::vector<Geom>& gs, int* doff, cudaStream_t st
   B.fam_time = doff + fam_at + count;
   B.filt = nullptr;
   B.filt_want = 0;
-  CK(cudaMemcpyAsync(doff + fam_at, staging.data() + fam_at, 2 * count * sizeof(int), cudaMemcpyHostToDevice, st));
+  for (int p = 0; p < 2; ++p) {
+    B.lane_sp[p] = doff + staging.size();
+    for (const Geom& g : gs) staging.push_back(g.lane_sp[p]);
+    B.lane_tm[p] = doff + staging.size();
+    for (const Geom& g : gs) staging.push_back(g.lane_tm[p]);
+    B.lane_sp_set[p] = B.lane_tm_set[p] = 0;
+    for (const Geom& g : gs) {
+      if (g.ls_blocks[p] > 0) B.lane_sp_set[p] |= 1u << g.lane_sp[p];
+      if (g.lt_blocks[p] > 0) B.lane_tm_set[p] |= 1u << g.lane_tm[p];
+    }
+  }
+  CK(cudaMemcpyAsync(doff + fam_at, staging.data() + fam_at, (staging.size() - fam_at) * sizeof(int),
+                     cudaMemcpyHostToDevice, st));
   return PCB_OK;
 }
 }  // namespace pcb
@@ -429,6 +473,9 @@ int validate_desc(const pcb_desc* d) {
   return PCB_OK;
 }
 
+// launch shapes after a change of the kernel choices (Geom::tune)
+void reshape_geom(Geom& g) { set_shapes(g); }
+
 // Scalar fields, FFT plans and launch shapes of a validated descriptor (no device work).
 void init_geom(const pcb_desc* d, Geom& g) {
   std::memset(&g, 0, sizeof(g));
@@ -460,7 +507,7 @@ size_t table_layout(const Geom& g, TableLayout& t) {
   auto take = [&](size_t bytes) { size_t o = off_b; off_b += (bytes + 255) & ~(size_t)255; return o; };
   t.kap = take((size_t)N * 8); t.mud = take((size_t)n * 16); t.muf = take((size_t)n * 8);
   t.twdd = take((size_t)M * 16); t.twdf = take((size_t)M * 8); t.twtd = take((size_t)n * 16);
-  t.twtf = take((size_t)n * 8); t.pred = take((size_t)n * 16); t.pref = take((size_t)n * 8);
+  t.twtf = take((size_t)n * 8); t.pred = take((size_t)2 * n * 16); t.pref = take((size_t)2 * n * 8);
   t.ax = take(ne * 8); t.ay = take(ne * 8); t.dg = take(g.var_a ? (size_t)g.m * 8 : 0);
   t.ms = take(g.fem ? (size_t)N * 8 : 0);
   t.bytes = off_b;
@@ -513,7 +560,7 @@ void fill_tables(const pcb_desc* d, const Geom& g, const TableLayout& t, unsigne
   fill_tw((double2*)(host + t.twtd), (float2*)(host + t.twtf), n);
   double2* pred = (double2*)(host + t.pred);
   float2* pref = (float2*)(host + t.pref);
-  for (int k = 0; k < n; ++k) {
+  for (int k = 0; k < 2 * n; ++k) {
     const double a = (g.zeta_pi ? -M_PI : -g.zeta) * (double)k / n;   // exp(-i zeta t / n)
     pred[k].x = std::cos(a); pred[k].y = std::sin(a);
     pref[k].x = (float)pred[k].x; pref[k].y = (float)pred[k].y;
@@ -600,7 +647,7 @@ int pcb_create(const pcb_desc* d_in, pcb_problem** out) {
   }
   // ---- single-instance batch ----
   if (cudaMalloc(&p->dG, sizeof(Geom)) != cudaSuccess || cudaMalloc(&p->dS, sizeof(Slots)) != cudaSuccess ||
-      cudaMalloc(&p->dSc, sizeof(Scal)) != cudaSuccess || cudaMalloc(&p->doff, 10 * 2 * sizeof(int)) != cudaSuccess ||
+      cudaMalloc(&p->dSc, sizeof(Scal)) != cudaSuccess || cudaMalloc(&p->doff, batch_ints(1) * sizeof(int)) != cudaSuccess ||
       cudaMalloc(&p->partial, (size_t)g.vec_blocks * (PCB_MAX_RESTART + 2) * sizeof(double) +
                                   (size_t)std::max(g.mv_blocks, 1) * sizeof(double)) != cudaSuccess)
     return fail(PCB_ERR_OUT_OF_MEMORY);
@@ -1218,6 +1265,7 @@ bool tune_valid(const Geom& g0, TuneChoice c, int prec) {
   Geom g = g0;
   apply_choice(g, c);
   const int pr = prec == PCB_MIXED ? 1 : 0;
+  if (g.lane_sp[pr]) return true;
   const bool pipe_d = pr && pipe_dst_p(g), pipe_t = pr && pipe_time_p(g);
   if (!pipe_d && dst_smem_bytes(g, pr) > kSmemMax) return false;
   if (!pipe_t && time_smem_bytes(g, pr) > kSmemMax) return false;
@@ -1237,22 +1285,25 @@ std::vector<TuneChoice> tune_candidates(const Geom& g, int prec) {
     if (tune_valid(g, c, prec)) out.push_back(c);
   };
   add(0, q0d, q0t);                                   // the default shapes come first
+  // then the other kernels' shapes, without the one-line-per-lane passes where the default takes them
   Geom d = g;
-  apply_choice(d, out.empty() ? TuneChoice{0, q0d, q0t} : out[0]);
+  const int nl = [&] { Geom t = g; apply_choice(t, TuneChoice{0, q0d, q0t}); return t.lane_sp[prec == PCB_MIXED] ? TUNE_NO_LANE : 0; }();
+  if (nl) add(nl, q0d, q0t);
+  apply_choice(d, TuneChoice{nl, q0d, q0t});
   const bool mixed = prec == PCB_MIXED;
   const bool can_pipe_t = mixed && pipe_time_p(d), can_pipe_d = mixed && pipe_dst_p(d);
-  if (can_pipe_d && can_pipe_t && g.n == 512) add(TUNE_NO_HANDOFF, q0d, q0t);
+  if (can_pipe_d && can_pipe_t && g.n == 512) add(nl | TUNE_NO_HANDOFF, q0d, q0t);
   if (can_pipe_t && g.n == 512 && g.zeta_pi) {
     for (int v : {TUNE_TIME512_3BLK, TUNE_TIME512_4BLK}) {
-      add(v, q0d, q0t);
-      if (can_pipe_d) add(v | TUNE_NO_HANDOFF, q0d, q0t);
+      add(nl | v, q0d, q0t);
+      if (can_pipe_d) add(nl | v | TUNE_NO_HANDOFF, q0d, q0t);
     }
   }
   for (int b = 0; b < 3; ++b) {
     const int bs = b << 4;
     for (int dq : qd) {
-      if (can_pipe_t) add(TUNE_NO_PIPE_DST | bs, dq, q0t);          // tile spatial passes, pipelined time
-      for (int tq : qt) add(TUNE_NO_PIPE_DST | TUNE_NO_PIPE_TIME | bs, dq, tq);   // tile kernels only
+      if (can_pipe_t) add(nl | TUNE_NO_PIPE_DST | bs, dq, q0t);     // tile spatial passes, pipelined time
+      for (int tq : qt) add(nl | TUNE_NO_PIPE_DST | TUNE_NO_PIPE_TIME | bs, dq, tq);   // tile kernels only
     }
   }
   return out;
@@ -1260,9 +1311,10 @@ std::vector<TuneChoice> tune_candidates(const Geom& g, int prec) {
 
 // the configuration a problem runs, in the terms of pcb_tune_info
 void describe_choice(const Geom& g, int prec, pcb_tune_info* info) {
-  info->pipelined_dst = prec == PCB_MIXED && pipe_dst_p(g);
-  info->pipelined_time = prec == PCB_MIXED && pipe_time_p(g);
-  info->time_major_handoff = prec == PCB_MIXED && (pipe_dst_code(g) & 64) ? 1 : 0;
+  const bool ln = g.lane_sp[prec == PCB_MIXED] != 0;      // neither pipelined nor tile kernels
+  info->pipelined_dst = !ln && prec == PCB_MIXED && pipe_dst_p(g);
+  info->pipelined_time = !ln && prec == PCB_MIXED && pipe_time_p(g);
+  info->time_major_handoff = !ln && prec == PCB_MIXED && (pipe_dst_code(g) & 64) ? 1 : 0;
   info->dst_lanes = g.M / g.dst_q;
   info->time_lanes = g.n / g.time_q;
   info->tile_scale = tune_budget_shift(g.tune) == 1 ? 0.5 : tune_budget_shift(g.tune) == 2 ? 2.0 : 1.0;
@@ -1564,7 +1616,7 @@ int group_setup(BGroup& G, const SolveCfg& c, const double* const* b_dev, double
   part = std::max((size_t)tv * (PCB_MAX_RESTART + 1), (size_t)tm) + 1;
   if (cudaMalloc(&G.dG, sizeof(Geom) * n) || cudaMalloc(&G.dS, sizeof(Slots) * n) ||
       cudaMalloc(&G.dSc, sizeof(Scal) * n) || cudaMalloc(&G.dAct, sizeof(int) * n) ||
-      cudaMalloc(&G.dOff, sizeof(int) * 10 * (n + 1)) || cudaMalloc(&G.dPart, part * sizeof(double)) ||
+      cudaMalloc(&G.dOff, sizeof(int) * batch_ints(n)) || cudaMalloc(&G.dPart, part * sizeof(double)) ||
       cudaMalloc(&G.dTol, sizeof(double) * n) || cudaMallocHost(&G.hSc, sizeof(Scal) * n) ||
       cudaMallocHost(&G.hAct, sizeof(int) * n) || cudaMallocHost(&G.hTol, sizeof(double) * n)) {
     cudaGetLastError();
@@ -2219,7 +2271,7 @@ int pcb_server_create(const pcb_server_opts* o, pcb_server** out) {
     const size_t part = (size_t)n * 2432 * (PCB_MAX_RESTART + 1) + 1;
     if (cudaMalloc(&G.dG, sizeof(Geom) * n) || cudaMalloc(&G.dS, sizeof(Slots) * n) ||
         cudaMalloc(&G.dSc, sizeof(Scal) * n) || cudaMalloc(&G.dAct, sizeof(int) * n) ||
-        cudaMalloc(&G.dOff, sizeof(int) * 10 * (n + 1)) || cudaMalloc(&G.dPart, part * sizeof(double)) ||
+        cudaMalloc(&G.dOff, sizeof(int) * batch_ints(n)) || cudaMalloc(&G.dPart, part * sizeof(double)) ||
         cudaMalloc(&G.dTol, sizeof(double) * n) || cudaMallocHost(&G.hSc, sizeof(Scal) * n) ||
         cudaMallocHost(&G.hAct, sizeof(int) * n) || cudaMallocHost(&G.hTol, sizeof(double) * n) ||
         cudaMallocHost(&G.hSpin, sizeof(Slots) * n)) {
