@@ -94,9 +94,9 @@ __device__ __forceinline__ Epi make_epi(int kind, const Scal* sc) {
 }
 
 // Blocks of kMvThreads threads, one spatial column per thread.  theta == 1: blocks =
-// ceil(m/kMvThreads) * ceil(n/tchunk) (fused); else blocks = 2 * ceil(m/kMvThreads) (forward-marching
-// T role, backward-marching T^T role), each thread marching over all n time steps.  The marching
-// form has only 2m threads, so the block is small enough that they all fit on the device at once:
+// ceil(m/kMvThreads) * ceil(n/tchunk) (fused); else blocks = 2 * ceil(m mv_chunks/kMvThreads) (forward-marching
+// T role, backward-marching T^T role), each thread marching over n / mv_chunks time steps.  The marching
+// form of a large grid has only 2m threads, so the block is small enough that they all fit on the device at once:
 // with 256-thread blocks a problem of m = 66,049 columns needed a second wave of 62 blocks, which
 // took as long as the first.
 constexpr int kMvThreads = 128;
@@ -115,8 +115,95 @@ void matvec_shape(Geom& g) {
     g.mv_blocks = units * ((g.n + tch - 1) / tch);
   } else {
     g.mv_tchunk = g.n;
-    g.mv_blocks = 2 * ncb;
+    // march_block: parts of the time range while that leaves at least four steps each and the device
+    // short of threads (about 250 a multiprocessor, half of what it holds at this register count; with
+    // more columns the extra operation of the first sweep costs more than the threads give)
+    g.mv_chunks = 1;
+    while (g.mv_chunks < 8 && g.n / (2 * g.mv_chunks) >= 4 && 2LL * g.m * g.mv_chunks < 76000) g.mv_chunks *= 2;
+    const int cpb = kMvThreads / g.mv_chunks;
+    g.mv_blocks = 2 * ((g.m + cpb - 1) / cpb);
   }
+}
+
+// theta < 1, one role of one block of columns: T x1 - alpha x2 marching forward in time (role 0) or
+// alpha x1 + T^T x2 marching backward (role 1).  With u the marched half, the recurrence
+// z_t = (u_t - (1-theta) z_{t-1})/theta gives (B_n u)_t = z_t - z_{t-1} = (u_t - z_{t-1})/theta, so
+//     out = (1/theta + diagonal) u_t - z_{t-1}/theta - (off-diagonal sum) -/+ alpha (other half)
+// and, for theta = 1/2, z_t = 2 u_t - z_{t-1}: eight FP64 operations per value for a constant
+// coefficient (ten when the difference z_t - z_{t-1} and the stencil are formed on their own).  The
+// kernel is bound by FP64 issue: N = 255, n = 256 0.84 -> 0.70 ms, 72% of the measured FP64 rate.
+// A small grid has too few columns to fill the device with one thread each.  Its time range is split
+// in g.mv_chunks parts: a first sweep marches every part from z = 0, the carries combine through
+// (-(1-theta)/theta)^length, and the second sweep computes the values (GMRES
+// solve at N = 63, n = 64: 2.71 -> 2.28 ms, its products having taken 84 us each).
+template <bool VAR>
+__device__ __forceinline__ double march_block(const Geom& g, int lb, int op, const double* __restrict__ x,
+                                              double* __restrict__ out, const double* __restrict__ aux, const Epi& e) {
+  __shared__ double carry[kMvThreads];
+  const int N = g.N, m = g.m, n = g.n, chunks = g.mv_chunks, cpb = kMvThreads / chunks;
+  const long long mn = g.mn;
+  const int ncb = (m + cpb - 1) / cpb;
+  const int role = lb / ncb, ch = threadIdx.x / cpb, cl = threadIdx.x - ch * cpb;
+  const int col = (lb - role * ncb) * cpb + cl;
+  const bool ok = col < m;
+  const int len = n / chunks, s0 = ch * len;               // n and chunks are powers of two
+  const int t0 = role ? n - 1 - s0 : s0;
+  const long long step = role ? -(long long)m : m;
+  const double th = g.theta, ith = 1.0 / th, r = (1.0 - th) * ith;
+  const bool half = r == 1.0;                              // theta = 1/2
+  const long long at0 = (long long)t0 * m + (ok ? col : 0);
+  const double* __restrict__ u = x + (role ? mn : 0) + at0;
+  double z = 0.0;
+  if (chunks > 1) {
+    const double* v = u;
+    if (ok)
+      for (int k = 0; k < len; ++k, v += step) z = half ? fma(ith, *v, -z) : fma(-r, z, ith * *v);
+    carry[threadIdx.x] = z;
+    __syncthreads();
+    double pw = 1.0;
+    for (int k = 0; k < len; ++k) pw *= -r;
+    z = 0.0;
+    for (int c = 0; c < ch; ++c) z = fma(pw, z, carry[c * cpb + cl]);
+  }
+  double part = 0.0;
+  if (!ok) return part;
+  const int j = col / N, i = col - j * N;
+  const bool neu = g.bc == PCB_BC_NEUMANN;
+  // neighbour offsets: the mirrored neighbour at a Neumann boundary, masked to zero at a Dirichlet one
+  const int oL = i > 0 ? -1 : (neu ? 1 : 0), oR = i < N - 1 ? 1 : (neu ? -1 : 0);
+  const int oD = j > 0 ? -N : (neu ? N : 0), oU = j < N - 1 ? N : (neu ? -N : 0);
+  const double alpha = role ? g.alpha : -g.alpha;
+  double kc, kL = 0.0, kR = 0.0, kD = 0.0, kU = 0.0;
+  if (VAR) {
+    const double* ax = g.axs + (long long)j * (N + 1) + i;
+    kL = oL ? -ax[0] : 0.0; kR = oR ? -ax[1] : 0.0;
+    kD = oD ? -g.ays[col] : 0.0; kU = oU ? -g.ays[col + N] : 0.0;
+    kc = ith + g.dgs[col];
+  } else {
+    kc = fma(4.0, g.c, ith);
+  }
+  const long long offs = (role == 0) == (op == PCB_OP_A) ? mn : 0;
+  const double* __restrict__ w = x + (role ? 0 : mn) + at0;
+  long long a = offs + at0;
+#pragma unroll 2
+  for (int k = 0; k < len; ++k, u += step, w += step, a += step) {
+    const double uc = *u;
+    const double l = oL ? u[oL] : 0.0, rr = oR ? u[oR] : 0.0, d = oD ? u[oD] : 0.0, t = oU ? u[oU] : 0.0;
+    double o;
+    if (VAR) {
+      o = fma(kL, l, kc * uc);
+      o = fma(kR, rr, o);
+      o = fma(kD, d, o);
+      o = fma(kU, t, o);
+    } else {
+      o = fma(-g.c, (l + rr) + (d + t), kc * uc);
+    }
+    o = fma(-ith, z, o);
+    o = fma(alpha, *w, o);
+    z = half ? fma(ith, uc, -z) : fma(-r, z, ith * uc);
+    out[a] = epi_apply(e, o, aux, x, a, part);
+  }
+  return part;
 }
 
 // The FP64 product of block lb of one instance with its epilogue; returns the block's epilogue
@@ -222,55 +309,48 @@ __device__ __forceinline__ double matvec_block(const Geom& g, int lb, int op, co
         x1prev = x1c;
       }
     }
-  } else {
-    const int role = lb / ncb, cb = lb - role * ncb;
-    const int col = cb * kMvThreads + threadIdx.x;
-    if (col < m) {
-      const int j = col / N, i = col - j * N;
-      const double th = g.theta, om = 1.0 - th, ith = 1.0 / th;
-      if (role == 0) {
-        // forward: z_t = (x1_t - (1-theta) z_{t-1})/theta, (B_n x1)_t = z_t - z_{t-1}
-        double zprev = 0.0;
-#pragma unroll 2
-        for (int t = 0; t < n; ++t) {
-          const long long a = (long long)t * m + col;
-          const double* u1 = x1 + (long long)t * m;
-          const double z = fma(-om, zprev, u1[col]) * ith;
-          double oT = (z - zprev) + tauK(g, u1, i, j, col);
-          oT = fma(-alpha, x2[a], oT);
-          out[offT + a] = epi_apply(e, oT, aux, x, offT + a, part);
-          zprev = z;
-        }
-      } else {
-        // backward: u_t = (x2_t - (1-theta) u_{t+1})/theta, (B_n^T x2)_t = u_t - u_{t+1}
-        double unext = 0.0;
-#pragma unroll 2
-        for (int t = n - 1; t >= 0; --t) {
-          const long long a = (long long)t * m + col;
-          const double* u2 = x2 + (long long)t * m;
-          const double u = fma(-om, unext, u2[col]) * ith;
-          double oTT = (u - unext) + tauK(g, u2, i, j, col);
-          oTT = fma(alpha, x1[a], oTT);
-          out[offTT + a] = epi_apply(e, oTT, aux, x, offTT + a, part);
-          unext = u;
-        }
-      }
-    }
   }
   if (epi_kind == EPI_MINRES) part *= e.s;
   return part;
 }
 
+// Which of the three product kernels an instance takes: a launch of one covers the whole block range
+// and skips the instances of the others (launch_matvec issues those that are present).
+enum { MV_STEP = 1, MV_MARCH = 2, MV_TW = 4 };
+__device__ __forceinline__ int matvec_kernel(const Geom& g, int fast) {
+  return g.theta != 1.0 ? MV_MARCH : (fast && !g.var_a ? MV_TW : MV_STEP);
+}
+
 __global__ void __launch_bounds__(kMvThreads) k_matvec(const Geom* __restrict__ G, const Slots* __restrict__ S,
+                                                Scal* __restrict__ Sc, const int* __restrict__ off, int count,
+                                                const int* __restrict__ active, int op, int x_slot, int out_slot,
+                                                int aux_slot, int epi_kind, int fast, double* __restrict__ partial) {
+  const int inst = find_inst(off, count, blockIdx.x);
+  if (active && !active[inst]) return;
+  const Geom& g = G[inst];
+  if (matvec_kernel(g, fast) != MV_STEP) return;
+  const double* __restrict__ aux = aux_slot >= 0 ? S[inst].v[aux_slot] : nullptr;
+  const double part = matvec_block(g, blockIdx.x - off[inst], op, S[inst].v[x_slot], S[inst].v[out_slot], aux,
+                                   make_epi(epi_kind, Sc + inst), epi_kind);
+  if (partial && epi_kind != EPI_PLAIN) block_reduce_store(part, partial + blockIdx.x);
+}
+
+// seven blocks an SM: the columns of a 257 x 257 grid in one wave
+__global__ void __launch_bounds__(kMvThreads, 7) k_matvec_march(const Geom* __restrict__ G, const Slots* __restrict__ S,
                                                 Scal* __restrict__ Sc, const int* __restrict__ off, int count,
                                                 const int* __restrict__ active, int op, int x_slot, int out_slot,
                                                 int aux_slot, int epi_kind, double* __restrict__ partial) {
   const int inst = find_inst(off, count, blockIdx.x);
   if (active && !active[inst]) return;
   const Geom& g = G[inst];
+  if (matvec_kernel(g, 0) != MV_MARCH) return;
   const double* __restrict__ aux = aux_slot >= 0 ? S[inst].v[aux_slot] : nullptr;
-  const double part = matvec_block(g, blockIdx.x - off[inst], op, S[inst].v[x_slot], S[inst].v[out_slot], aux,
-                                   make_epi(epi_kind, Sc + inst), epi_kind);
+  const Epi e = make_epi(epi_kind, Sc + inst);
+  const int lb = blockIdx.x - off[inst];
+  const double* __restrict__ x = S[inst].v[x_slot];
+  double* __restrict__ out = S[inst].v[out_slot];
+  double part = g.var_a ? march_block<true>(g, lb, op, x, out, aux, e) : march_block<false>(g, lb, op, x, out, aux, e);
+  if (epi_kind == EPI_MINRES) part *= e.s;
   if (partial && epi_kind != EPI_PLAIN) block_reduce_store(part, partial + blockIdx.x);
 }
 
@@ -570,12 +650,11 @@ __global__ void __launch_bounds__(kMvThreads) k_matvec_tw(const Geom* __restrict
   const int inst = find_inst(off, count, blockIdx.x);
   if (active && !active[inst]) return;
   const Geom& g = G[inst];
+  if (matvec_kernel(g, 1) != MV_TW) return;
   const double* __restrict__ aux = aux_slot >= 0 ? S[inst].v[aux_slot] : nullptr;
   const Epi e = make_epi(EPI_MINRES, Sc + inst);
   const int lb = blockIdx.x - off[inst];
-  const double part = (g.theta == 1.0 && !g.var_a)
-                          ? matvec_tw_block(g, lb, op, S[inst].v[x_slot], S[inst].v[out_slot], aux, e, Sc[inst], tile)
-                          : matvec_block(g, lb, op, S[inst].v[x_slot], S[inst].v[out_slot], aux, e, EPI_MINRES);
+  const double part = matvec_tw_block(g, lb, op, S[inst].v[x_slot], S[inst].v[out_slot], aux, e, Sc[inst], tile);
   if (partial) block_reduce_store(part, partial + blockIdx.x);
 }
 
@@ -610,15 +689,22 @@ cudaError_t launch_matvec(const Batch& B, int op, int x_slot, int out_slot, int 
                                                    B.partial);
     return cudaGetLastError();
   }
-  if ((epi & EPI_FAST) && (epi & (EPI_FAST - 1)) == EPI_MINRES) {
+  const int kind = epi & (EPI_FAST - 1), fast = (epi & EPI_FAST) && kind == EPI_MINRES;
+  const int set = fast ? B.mv_set_fast : B.mv_set;
+  if (set & MV_TW)
     k_matvec_tw<<<B.tot_mv, kMvThreads, 0, B.stream>>>(B.G, B.S, B.Sc, B.off_mv, B.count, B.active, op, x_slot,
                                                        out_slot, aux_slot, B.partial);
-    return cudaGetLastError();
-  }
-  k_matvec<<<B.tot_mv, kMvThreads, 0, B.stream>>>(B.G, B.S, B.Sc, B.off_mv, B.count, B.active, op, x_slot, out_slot,
-                                           aux_slot, epi & (EPI_FAST - 1), B.partial);
+  if (set & MV_MARCH)
+    k_matvec_march<<<B.tot_mv, kMvThreads, 0, B.stream>>>(B.G, B.S, B.Sc, B.off_mv, B.count, B.active, op, x_slot,
+                                                          out_slot, aux_slot, kind, B.partial);
+  if (set & MV_STEP)
+    k_matvec<<<B.tot_mv, kMvThreads, 0, B.stream>>>(B.G, B.S, B.Sc, B.off_mv, B.count, B.active, op, x_slot, out_slot,
+                                                    aux_slot, kind, fast, B.partial);
   return cudaGetLastError();
 }
+
+// the product kernels an instance needs: MV_* of the FP64 product, or of the two-word one (fast)
+int matvec_kernel_of(const Geom& g, int fast) { return g.theta != 1.0 ? MV_MARCH : (fast && !g.var_a ? MV_TW : MV_STEP); }
 
 // ------------------------------------------------------------------------------------------
 // Right-hand side (Sec. 1: f~, g~ with M = I, then [g; sqrt(gamma) f] or [sqrt(gamma) f; g]).

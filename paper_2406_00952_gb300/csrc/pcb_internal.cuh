@@ -143,6 +143,7 @@ struct Geom {
   int ls_blocks[2], lt_blocks[2];
   int tune;                       // kernel choices of the autotuner (TUNE_* bits; 0 = defaults)
   int mv_tchunk;                  // time steps per thread in the theta = 1 matvec
+  int mv_chunks;                  // parts of the time range in the theta < 1 matvec
   int mv_blocks;                  // blocks of the matvec
   int vec_blocks;                 // blocks of the vector kernels over 2mn
   FftPlan pdst, ptime;
@@ -271,6 +272,7 @@ struct Batch {
   const int* off_time[2];  int tot_time[2];
   const int* off_ls[2];    int tot_ls[2];      // one-line-per-lane spatial and time passes
   const int* off_lt[2];    int tot_lt[2];
+  int mv_set, mv_set_fast;      // product kernels of the instances (matvec.cu), FP64 and two-word products
   const int* off_mv;    int tot_mv;
   const int* off_vec;   int tot_vec;
   double* partial;        // reduction partials

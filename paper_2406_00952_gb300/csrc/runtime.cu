@@ -64,6 +64,7 @@ cudaError_t launch_swap(const Batch& B, int a0, int b0, int a1, int b1, int a2, 
 cudaError_t launch_setslot(const Batch& B, int dst, int base, int k, int per_j = 0);
 size_t mg_workspace_bytes(const Geom& g);
 void matvec_shape(Geom& g);
+int matvec_kernel_of(const Geom& g, int fast);
 bool mg_available();
 int dst_Q(int N);
 int time_Q(int n);
@@ -327,6 +328,12 @@ int fill_batch(Batch& B, const std::vector<Geom>& gs, int* doff, cudaStream_t st
     }
   }
   B.off_mv = doff + 6 * stride; B.tot_mv = tots[6];
+  B.mv_set = B.mv_set_fast = 0;
+  for (const Geom& g : gs)
+    if (g.mv_blocks > 0) {
+      B.mv_set |= matvec_kernel_of(g, 0);
+      B.mv_set_fast |= matvec_kernel_of(g, 1);
+    }
   B.off_vec = doff + 7 * stride; B.tot_vec = tots[7];
   B.count = count;
   B.stream = st;
