@@ -106,59 +106,122 @@ __global__ void __launch_bounds__(256) k_minres_wx(const Geom* __restrict__ G, c
   }
 }
 
-// CGS: partial[blk*(PCB_MAX_RESTART+1) + i] = V_i . W,  i = 0..j.  JB >= j + 1 bounds the unrolled
-// basis loop: the host picks the smallest of 2, 4, 8, 16, 33 that covers the Arnoldi index, so an
-// early step does not pay for 33 predicated basis vectors per element.
-template <int JB>
-__global__ void __launch_bounds__(256) k_multidot(const Geom* __restrict__ G, const Slots* __restrict__ S,
+// Classical Gram-Schmidt over JB basis vectors, two values per thread and step (vectors have even
+// length and basis vectors start on 16 bytes).  Both kernels are bound by FP64 issue (one FMA per value
+// and vector: 63 us a vector at N = 255, n = 256, against 39 us of HBM) as long as enough loads are in
+// flight: the basis values of a step are loaded in groups of eight before they are used, and the blocks
+// per SM divide the 16 per SM of a large vector.  JB is the exact count (EXACT; a predicated-off step
+// costs its issue slot) or a bound on the per-instance count.  With one value per step and the loads left
+// to the compiler, 10, 12, 15 and 17-20 vectors ran 1.2-1.5 times above that rate (12 vectors 1.18 ms).
+constexpr int kGroup = 8;
+constexpr int gs_blocks(int JB) { return JB <= 8 ? 4 : 2; }
+
+// partial[i tot + blk] = V_i . W over the block's slice, i = 0 .. j
+template <int JB, bool EXACT>
+__global__ void __launch_bounds__(256, gs_blocks(JB)) k_multidot(const Geom* __restrict__ G, const Slots* __restrict__ S,
                                                   const Scal* __restrict__ Sc, const int* __restrict__ off, int count,
                                                   const int* __restrict__ active, int svbase, int j, int sw,
-                                                  double* __restrict__ partial) {
+                                                  double* __restrict__ partial, int tot) {
   INST_PROLOGUE
-  if (j < 0) j = Sc[inst].j;   // each instance at its own Arnoldi index
-  const double* __restrict__ V = S[inst].v[svbase];
-  const double* __restrict__ W = S[inst].v[sw];
+  if (!EXACT && j < 0) j = Sc[inst].j;   // each instance at its own Arnoldi index
+  const long long h = len / 2;
+  const double2* __restrict__ V = (const double2*)S[inst].v[svbase];
+  const double2* __restrict__ W = (const double2*)S[inst].v[sw];
   double acc[JB];
 #pragma unroll
   for (int i = 0; i < JB; ++i) acc[i] = 0.0;
-  for (long long e = e0; e < len; e += stride) {
-    const double w = W[e];
+#pragma unroll(JB <= 4 ? 4 : 1)
+  for (long long e = e0; e < h; e += stride) {
+    const double2 w = W[e];
 #pragma unroll
-    for (int i = 0; i < JB; ++i)
-      if (i <= j) acc[i] = fma(V[(long long)i * len + e], w, acc[i]);
+    for (int i0 = 0; i0 < JB; i0 += kGroup) {
+      double2 v[kGroup];
+#pragma unroll
+      for (int i = 0; i < kGroup; ++i)
+        if (i0 + i < JB && (EXACT || i0 + i <= j)) v[i] = V[(i0 + i) * h + e];
+#pragma unroll
+      for (int i = 0; i < kGroup; ++i)
+        if (i0 + i < JB && (EXACT || i0 + i <= j)) acc[i0 + i] = fma(v[i].y, w.y, fma(v[i].x, w.x, acc[i0 + i]));
+    }
   }
+  // block sums, eight at a time: halving the values held per lane at each exchange costs 9 FP64 additions
+  // a warp for eight sums instead of 40
+  constexpr int NGRP = (JB + 7) / 8;
+  __shared__ double red[NGRP][8][8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int i = 0; i < JB; ++i) {
-    if (i > j) break;
-    const double r = block_sum(acc[i]);
-    if (threadIdx.x == 0) partial[(long long)blockIdx.x * (PCB_MAX_RESTART + 1) + i] = r;
+  for (int q = 0; q < NGRP; ++q) {
+    double v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = 8 * q + i < JB ? acc[8 * q + i < JB ? 8 * q + i : 0] : 0.0;
+#pragma unroll
+    for (int w = 4; w >= 1; w >>= 1) {           // lane bit 4 w selects the upper w of 2 w values
+      const bool up = lane & (4 * w);
+#pragma unroll
+      for (int i = 0; i < w; ++i) {
+        const double send = up ? v[i] : v[i + w], keep = up ? v[i + w] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * w);
+      }
+    }
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+    if ((lane & 3) == 0) red[q][warp][lane >> 2] = v[0];
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < JB; i += blockDim.x) {
+    if (!EXACT && i > j) break;
+    double r = 0.0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) r += red[i >> 3][w][i & 7];
+    partial[(long long)i * tot + blockIdx.x] = r;
   }
 }
 
-// W -= sum_i h_i V_i (coef from Scal.H[pass*(MAX+1) + i]) ; or X += sum_i y_i Z_i (pass = -1)
-template <int JB>
-__global__ void __launch_bounds__(256) k_multiaxpy(const Geom* __restrict__ G, const Slots* __restrict__ S,
+// W -= sum_i h_i V_i (coef from Scal.H[pass*(MAX+1) + i]) ; or X += sum_i y_i Z_i (pass = -1).  pass 1 (the
+// second projection) also leaves partial[blk] = sum of W^2 over the block's slice: the norm of the new
+// basis vector without another sweep.  X may be a caller's vector aligned to 8 bytes only.
+template <int JB, bool EXACT>
+__global__ void __launch_bounds__(256, gs_blocks(JB)) k_multiaxpy(const Geom* __restrict__ G, const Slots* __restrict__ S,
                                                    const Scal* __restrict__ Sc, const int* __restrict__ off, int count,
                                                    const int* __restrict__ active, int svbase, int j, int sw,
-                                                   int pass) {
+                                                   int pass, double* __restrict__ partial) {
   INST_PROLOGUE
   const Scal& c = Sc[inst];
-  if (j < 0) j = pass >= 0 ? c.j : c.j - 1;   // per-instance index (after Arnoldi, c.j = columns)
-  const double* __restrict__ V = S[inst].v[svbase];
+  if (!EXACT && j < 0) j = pass >= 0 ? c.j : c.j - 1;   // per-instance index (after Arnoldi, c.j = columns)
+  const long long h = len / 2;
+  const double2* __restrict__ V = (const double2*)S[inst].v[svbase];
   double* __restrict__ W = S[inst].v[sw];
   double coef[JB];
 #pragma unroll
   for (int i = 0; i < JB; ++i) {
-    double h = 0.0;
-    if (i <= j) h = pass >= 0 ? -c.H[pass * (PCB_MAX_RESTART + 1) + i] : c.y[i];
-    coef[i] = h;
+    double k = 0.0;
+    if (EXACT || i <= j) k = pass >= 0 ? -c.H[pass * (PCB_MAX_RESTART + 1) + i] : c.y[i];
+    coef[i] = k;
   }
-  for (long long e = e0; e < len; e += stride) {
-    double w = W[e];
+  double sq = 0.0;
+#pragma unroll(JB <= 4 ? 4 : 1)
+  for (long long e = e0; e < h; e += stride) {
+    double wx = W[2 * e], wy = W[2 * e + 1];
 #pragma unroll
-    for (int i = 0; i < JB; ++i)
-      if (i <= j) w = fma(coef[i], V[(long long)i * len + e], w);
-    W[e] = w;
+    for (int i0 = 0; i0 < JB; i0 += kGroup) {
+      double2 v[kGroup];
+#pragma unroll
+      for (int i = 0; i < kGroup; ++i)
+        if (i0 + i < JB && (EXACT || i0 + i <= j)) v[i] = V[(i0 + i) * h + e];
+#pragma unroll
+      for (int i = 0; i < kGroup; ++i)
+        if (i0 + i < JB && (EXACT || i0 + i <= j)) {
+          wx = fma(coef[i0 + i], v[i].x, wx);
+          wy = fma(coef[i0 + i], v[i].y, wy);
+        }
+    }
+    W[2 * e] = wx;
+    W[2 * e + 1] = wy;
+    if (pass == 1) sq = fma(wy, wy, fma(wx, wx, sq));
+  }
+  if (pass == 1) {
+    const double r = block_sum(sq);
+    if (threadIdx.x == 0) partial[blockIdx.x] = r;
   }
 }
 
@@ -218,48 +281,72 @@ __device__ void scalar_step(Scal& c, int step, double v, double tol, int j, int 
       if (!isfinite(v)) { c.flags |= 4; c.active = 0; }
       break;
     }
-    case SS_GMRES_ARNOLDI: {
-      // v = ||w||^2 after two CGS passes; column j of H = H[0][.] + H[1][.]
-      const int M1 = PCB_MAX_RESTART + 1;
-      double* col = c.R + (long long)j * M1;
-      for (int i = 0; i <= j; ++i) col[i] = c.H[i] + c.H[M1 + i];
-      const double hn = sqrt(v);
-      col[j + 1] = hn;
-      c.hnorm = hn;
-      for (int i = 0; i < j; ++i) {
-        const double t = c.gcs[i] * col[i] + c.gsn[i] * col[i + 1];
-        col[i + 1] = -c.gsn[i] * col[i] + c.gcs[i] * col[i + 1];
-        col[i] = t;
-      }
-      double cs = 1.0, sn = 0.0;
-      if (col[j + 1] != 0.0) {
-        const double r = hypot(col[j], col[j + 1]);
-        cs = col[j] / r; sn = col[j + 1] / r;
-      }
-      c.gcs[j] = cs; c.gsn[j] = sn;
-      col[j] = cs * col[j] + sn * col[j + 1];
-      col[j + 1] = 0.0;
-      c.g[j + 1] = -sn * c.g[j];
-      c.g[j] = cs * c.g[j];
-      c.itn += 1;
-      c.j = j + 1;
-      c.est = fabs(c.g[j + 1]) / c.bnorm;
-      if (c.est <= tol) c.flags |= 1;
-      if (hn == 0.0) c.flags |= 8;        // lucky breakdown: the cycle ends here
-      if (!isfinite(c.est)) { c.flags |= 4; c.active = 0; }
-      // back substitution for the cycle's coefficients (used when the cycle ends)
-      const int k = j + 1;
-      for (int i = k - 1; i >= 0; --i) {
-        double s = c.g[i];
-        for (int q = i + 1; q < k; ++q) s -= c.R[(long long)q * M1 + i] * c.y[q];
-        c.y[i] = s / c.R[(long long)i * M1 + i];
-      }
-      break;
-    }
     default:
       break;
   }
   (void)restart;
+}
+
+// Arnoldi column j of FGMRES from the two projections' coefficients and v = ||w||^2: the earlier
+// rotations, a new one, the residual estimate.  The block stages the operands in shared memory (one thread
+// walking them in global memory took 15-50 us a step, the back substitution it also ran each time included;
+// k_backsub now runs that once, when the cycle ends).
+__device__ void arnoldi_step(Scal& c, double v, double tol, int j) {
+  const int M1 = PCB_MAX_RESTART + 1;
+  __shared__ double col[PCB_MAX_RESTART + 1], cs_[PCB_MAX_RESTART], sn_[PCB_MAX_RESTART];
+  for (int i = threadIdx.x; i <= j; i += blockDim.x) {
+    col[i] = c.H[i] + c.H[M1 + i];
+    if (i < j) { cs_[i] = c.gcs[i]; sn_[i] = c.gsn[i]; }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const double hn = sqrt(v);
+    double next = col[0];
+    for (int i = 0; i < j; ++i) {
+      const double b = col[i + 1];
+      col[i] = cs_[i] * next + sn_[i] * b;
+      next = -sn_[i] * next + cs_[i] * b;
+    }
+    double cs = 1.0, sn = 0.0;
+    if (hn != 0.0) {
+      const double r = hypot(next, hn);
+      cs = next / r; sn = hn / r;
+    }
+    col[j] = cs * next + sn * hn;
+    c.hnorm = hn;
+    c.gcs[j] = cs; c.gsn[j] = sn;
+    const double gj = c.g[j], gn = -sn * gj;
+    c.g[j + 1] = gn;
+    c.g[j] = cs * gj;
+    c.itn += 1;
+    c.j = j + 1;
+    c.est = fabs(gn) / c.bnorm;
+    if (c.est <= tol) c.flags |= 1;
+    if (hn == 0.0) c.flags |= 8;        // lucky breakdown: the cycle ends here
+    if (!isfinite(c.est)) { c.flags |= 4; c.active = 0; }
+  }
+  __syncthreads();
+  double* R = c.R + (long long)j * M1;
+  for (int i = threadIdx.x; i <= j; i += blockDim.x) R[i] = col[i];
+  if (threadIdx.x == 0) R[j + 1] = 0.0;
+}
+
+// coefficients y of the cycle's update, R y = g: one warp per instance, a column of R per step
+__global__ void __launch_bounds__(32) k_backsub(int count, const int* __restrict__ active, Scal* Sc) {
+  const int inst = blockIdx.x;
+  if (inst >= count || (active && !active[inst])) return;
+  Scal& c = Sc[inst];
+  const int k = c.j, lane = threadIdx.x, M1 = PCB_MAX_RESTART + 1;
+  __shared__ double s[PCB_MAX_RESTART];
+  for (int i = lane; i < k; i += 32) s[i] = c.g[i];
+  for (int q = k - 1; q >= 0; --q) {
+    __syncwarp();
+    const double* R = c.R + (long long)q * M1;
+    const double y = s[q] / R[q];
+    __syncwarp();
+    for (int i = lane; i < q; i += 32) s[i] -= R[i] * y;
+    if (lane == 0) c.y[q] = y;
+  }
 }
 
 // Sum the instance's partials (nper values per block, index `which`) and run a scalar step.
@@ -274,25 +361,31 @@ __global__ void __launch_bounds__(256) k_reduce(const int* __restrict__ off, int
   double acc = 0.0;
   for (int b = b0 + threadIdx.x; b < b1; b += blockDim.x) acc += partial[(long long)b * nper + which];
   const double s = block_sum(acc);
-  if (threadIdx.x == 0) scalar_step(Sc[inst], step, s, tols ? tols[inst] : tol, j < 0 ? Sc[inst].j : j, restart);
+  const double tl = tols ? tols[inst] : tol;
+  if (step == SS_GMRES_ARNOLDI) {
+    __shared__ double total;
+    if (threadIdx.x == 0) total = s;
+    __syncthreads();
+    arnoldi_step(Sc[inst], total, tl, j < 0 ? Sc[inst].j : j);
+  } else if (threadIdx.x == 0) {
+    scalar_step(Sc[inst], step, s, tl, j, restart);
+  }
 }
 
-// multi-reduction for CGS: H[pass][i] = sum of partials i
+// multi-reduction for CGS: H[pass][i] = sum of the partials of vector i = blockIdx.y (partial[i tot + b])
 __global__ void __launch_bounds__(256) k_reduce_multi(const int* __restrict__ off, int count,
                                                       const int* __restrict__ active,
-                                                      const double* __restrict__ partial, int j, int pass, Scal* Sc) {
-  const int inst = blockIdx.x;
+                                                      const double* __restrict__ partial, int tot, int j, int pass,
+                                                      Scal* Sc) {
+  const int inst = blockIdx.x, i = blockIdx.y;
   if (inst >= count) return;
   if (active && !active[inst]) return;
-  if (j < 0) j = Sc[inst].j;
+  if (i > (j < 0 ? Sc[inst].j : j)) return;
   const int b0 = off[inst], b1 = off[inst + 1];
-  for (int i = 0; i <= j; ++i) {
-    double acc = 0.0;
-    for (int b = b0 + threadIdx.x; b < b1; b += blockDim.x)
-      acc += partial[(long long)b * (PCB_MAX_RESTART + 1) + i];
-    const double s = block_sum(acc);
-    if (threadIdx.x == 0) Sc[inst].H[pass * (PCB_MAX_RESTART + 1) + i] = s;
-  }
+  double acc = 0.0;
+  for (int b = b0 + threadIdx.x; b < b1; b += blockDim.x) acc += partial[(long long)i * tot + b];
+  const double s = block_sum(acc);
+  if (threadIdx.x == 0) Sc[inst].H[pass * (PCB_MAX_RESTART + 1) + i] = s;
 }
 
 // swap slot pointers (per instance, one thread)
@@ -307,15 +400,15 @@ __global__ void k_swap(Slots* S, int count, const int* __restrict__ active, int 
   if (a2 >= 0) { t = S[inst].v[a2]; S[inst].v[a2] = S[inst].v[b2]; S[inst].v[b2] = t; }
 }
 
-// set slot `dst` = slot `base` + k * 2mn  (GMRES basis addressing); per_j: k is an offset from
-// the instance's own Arnoldi index
-__global__ void k_setslot(const Geom* __restrict__ G, Slots* S, const Scal* __restrict__ Sc, int count,
-                          const int* __restrict__ active, int dst, int base, int k, int per_j) {
+// GMRES basis addressing: slot `dst` = slot `base` + k * 2mn, for up to three (dst, base, k); dst < 0: none
+struct SetSlots { int dst[3], base[3], k[3]; };
+__global__ void k_setslot(const Geom* __restrict__ G, Slots* S, int count, const int* __restrict__ active, SetSlots q) {
   const int inst = blockIdx.x * blockDim.x + threadIdx.x;
   if (inst >= count) return;
   if (active && !active[inst]) return;
-  const int kk = per_j ? Sc[inst].j + k : k;
-  S[inst].v[dst] = S[inst].v[base] + (long long)kk * 2 * G[inst].mn;
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+    if (q.dst[a] >= 0) S[inst].v[q.dst[a]] = S[inst].v[q.base[a]] + (long long)q.k[a] * 2 * G[inst].mn;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -339,53 +432,75 @@ cudaError_t launch_minres_wx(const Batch& B, int sy, int sw, int sw2, int sx) {
   k_minres_wx<<<B.tot_vec, 256, 0, B.stream>>>(B.G, B.S, B.Sc, B.off_vec, B.count, B.active, sy, sw, sw2, sx);
   return cudaGetLastError();
 }
-// basis-loop bound for Arnoldi index j (j < 0: per-instance indices, at most jmax when jmax >= 0).
-// The loops are unrolled to the bound and predicated beyond j + 1; the kernels are bound by FP64
-// issue, so a predicated-off step still costs its slot: the bound is exact up to 20 basis vectors
-// and a multiple of 4 above (most solves stay in the exact range).
-static int basis_bound(int j, int jmax) {
-  if (j < 0) j = jmax;
-  const int need = j < 0 ? PCB_MAX_RESTART + 1 : j + 1;
-  if (need <= 20) return need < 1 ? 1 : need;
-  return need <= 24 ? 24 : need <= 28 ? 28 : PCB_MAX_RESTART + 1;
-}
-#define PCB_BASIS_BOUNDS(X)                                                                           \
-  X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12) X(13) X(14) X(15) X(16) X(17) X(18) \
-  X(19) X(20) X(24) X(28)
+// Arnoldi index j >= 0: the kernel of exactly j + 1 vectors.  j < 0 (per-instance indices, at most jmax when
+// jmax >= 0): the smallest bound that covers them.
+#define PCB_EXACT(X)                                                                                      \
+  X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12) X(13) X(14) X(15) X(16) X(17) X(18)     \
+  X(19) X(20) X(21) X(22) X(23) X(24) X(25) X(26) X(27) X(28) X(29) X(30) X(31) X(32) X(33)
+#define PCB_BOUNDS(X) X(2) X(4) X(6) X(8) X(10) X(12) X(14) X(16) X(20) X(24) X(33)
+static_assert(PCB_MAX_RESTART + 1 == 33, "the lists above end at the largest basis");
 cudaError_t launch_multidot(const Batch& B, int svbase, int j, int sw, int jmax) {
-#define PCB_MULTIDOT(JB) \
-  k_multidot<JB><<<B.tot_vec, 256, 0, B.stream>>>(B.G, B.S, B.Sc, B.off_vec, B.count, B.active, svbase, j, sw, B.partial)
-#define PCB_MULTIDOT_CASE(JB) case JB: PCB_MULTIDOT(JB); break;
-  switch (basis_bound(j, jmax)) {
-    PCB_BASIS_BOUNDS(PCB_MULTIDOT_CASE)
-    default: PCB_MULTIDOT(PCB_MAX_RESTART + 1); break;
+#define PCB_ARGS B.G, B.S, B.Sc, B.off_vec, B.count, B.active, svbase, j, sw, B.partial, B.tot_vec
+  if (j >= 0) {
+    switch (j + 1) {
+#define PCB_CASE(JB) case JB: k_multidot<JB, true><<<B.tot_vec, 256, 0, B.stream>>>(PCB_ARGS); break;
+      PCB_EXACT(PCB_CASE)
+#undef PCB_CASE
+      default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
   }
-#undef PCB_MULTIDOT_CASE
-#undef PCB_MULTIDOT
+  const int need = jmax < 0 ? PCB_MAX_RESTART + 1 : jmax + 1;
+#define PCB_CASE(JB) \
+  if (need <= JB) { k_multidot<JB, false><<<B.tot_vec, 256, 0, B.stream>>>(PCB_ARGS); return cudaGetLastError(); }
+  PCB_BOUNDS(PCB_CASE)
+#undef PCB_CASE
+#undef PCB_ARGS
+  return cudaErrorInvalidValue;
+}
+// jmax: as for launch_multidot
+cudaError_t launch_reduce_multi(const Batch& B, int j, int pass, int jmax) {
+  const int rows = j >= 0 ? j + 1 : jmax >= 0 ? jmax + 1 : PCB_MAX_RESTART + 1;
+  k_reduce_multi<<<dim3(B.count, rows), 256, 0, B.stream>>>(B.off_vec, B.count, B.active, B.partial, B.tot_vec, j, pass,
+                                                           B.Sc);
   return cudaGetLastError();
 }
-cudaError_t launch_reduce_multi(const Batch& B, int j, int pass) {
-  k_reduce_multi<<<B.count, 256, 0, B.stream>>>(B.off_vec, B.count, B.active, B.partial, j, pass, B.Sc);
+cudaError_t launch_backsub(const Batch& B) {
+  k_backsub<<<B.count, 32, 0, B.stream>>>(B.count, B.active, B.Sc);
   return cudaGetLastError();
 }
 cudaError_t launch_multiaxpy(const Batch& B, int svbase, int j, int sw, int pass, int jmax) {
-#define PCB_MULTIAXPY(JB) \
-  k_multiaxpy<JB><<<B.tot_vec, 256, 0, B.stream>>>(B.G, B.S, B.Sc, B.off_vec, B.count, B.active, svbase, j, sw, pass)
-#define PCB_MULTIAXPY_CASE(JB) case JB: PCB_MULTIAXPY(JB); break;
-  switch (basis_bound(j, jmax)) {
-    PCB_BASIS_BOUNDS(PCB_MULTIAXPY_CASE)
-    default: PCB_MULTIAXPY(PCB_MAX_RESTART + 1); break;
+#define PCB_ARGS B.G, B.S, B.Sc, B.off_vec, B.count, B.active, svbase, j, sw, pass, B.partial
+  if (j >= 0) {
+    switch (j + 1) {
+#define PCB_CASE(JB) case JB: k_multiaxpy<JB, true><<<B.tot_vec, 256, 0, B.stream>>>(PCB_ARGS); break;
+      PCB_EXACT(PCB_CASE)
+#undef PCB_CASE
+      default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
   }
-#undef PCB_MULTIAXPY_CASE
-#undef PCB_MULTIAXPY
-  return cudaGetLastError();
+  const int need = jmax < 0 ? PCB_MAX_RESTART + 1 : jmax + 1;
+#define PCB_CASE(JB) \
+  if (need <= JB) { k_multiaxpy<JB, false><<<B.tot_vec, 256, 0, B.stream>>>(PCB_ARGS); return cudaGetLastError(); }
+  PCB_BOUNDS(PCB_CASE)
+#undef PCB_CASE
+#undef PCB_ARGS
+  return cudaErrorInvalidValue;
 }
 cudaError_t launch_swap(const Batch& B, int a0, int b0, int a1, int b1, int a2, int b2) {
   k_swap<<<(B.count + 63) / 64, 64, 0, B.stream>>>(B.S, B.count, B.active, a0, b0, a1, b1, a2, b2);
   return cudaGetLastError();
 }
-cudaError_t launch_setslot(const Batch& B, int dst, int base, int k, int per_j) {
-  k_setslot<<<(B.count + 63) / 64, 64, 0, B.stream>>>(B.G, B.S, B.Sc, B.count, B.active, dst, base, k, per_j);
+cudaError_t launch_setslot(const Batch& B, int dst, int base, int k) {
+  const SetSlots q = {{dst, -1, -1}, {base, 0, 0}, {k, 0, 0}};
+  k_setslot<<<(B.count + 63) / 64, 64, 0, B.stream>>>(B.G, B.S, B.count, B.active, q);
+  return cudaGetLastError();
+}
+// the three vectors of Arnoldi step j: v_j, z_j, v_{j+1}
+cudaError_t launch_setslots(const Batch& B, int vj, int zj, int vj1, int vbase, int zbase, int j) {
+  const SetSlots q = {{vj, zj, vj1}, {vbase, zbase, vbase}, {j, j, j + 1}};
+  k_setslot<<<(B.count + 63) / 64, 64, 0, B.stream>>>(B.G, B.S, B.count, B.active, q);
   return cudaGetLastError();
 }
 

@@ -58,10 +58,12 @@ cudaError_t launch_axpby(const Batch& B, int mode, int sx, int sy, int sz);
 cudaError_t launch_minres_wx(const Batch& B, int sy, int sw, int sw2, int sx);
 // j < 0: each instance at its own Arnoldi index (from Scal), all of them <= jmax when jmax >= 0
 cudaError_t launch_multidot(const Batch& B, int svbase, int j, int sw, int jmax = -1);
-cudaError_t launch_reduce_multi(const Batch& B, int j, int pass);
+cudaError_t launch_reduce_multi(const Batch& B, int j, int pass, int jmax = -1);
+cudaError_t launch_backsub(const Batch& B);
 cudaError_t launch_multiaxpy(const Batch& B, int svbase, int j, int sw, int pass, int jmax = -1);
 cudaError_t launch_swap(const Batch& B, int a0, int b0, int a1, int b1, int a2, int b2);
-cudaError_t launch_setslot(const Batch& B, int dst, int base, int k, int per_j = 0);
+cudaError_t launch_setslot(const Batch& B, int dst, int base, int k);
+cudaError_t launch_setslots(const Batch& B, int vj, int zj, int vj1, int vbase, int zbase, int j);
 size_t mg_workspace_bytes(const Geom& g);
 void matvec_shape(Geom& g);
 int matvec_kernel_of(const Geom& g, int fast);
@@ -932,9 +934,7 @@ static int minres_single(pcb_problem* p, const SolveCfg& c, int s_b, int s_x, Sc
 static int arnoldi_launches(pcb_problem* p, const Batch& B, const SolveCfg& c, int j) {
   int rc;
   const int op = PCB_OP_AHAT;
-  CK(LC(p) launch_setslot(B, SL_VJ, SL_VBASE, j));
-  CK(LC(p) launch_setslot(B, SL_ZJ, SL_ZBASE, j));
-  CK(LC(p) launch_setslot(B, SL_VJ1, SL_VBASE, j + 1));
+  CK(LC(p) launch_setslots(B, SL_VJ, SL_ZJ, SL_VJ1, SL_VBASE, SL_ZBASE, j));
   if ((rc = P_precond(p, B, c.kind, c.prec, SL_VJ, SL_ZJ))) return rc;
   CK(P_matvec(p, B, op, SL_ZJ, SL_VJ1, -1, EPI_PLAIN));
   for (int pass = 0; pass < 2; ++pass) {
@@ -942,7 +942,6 @@ static int arnoldi_launches(pcb_problem* p, const Batch& B, const SolveCfg& c, i
     CK(LC(p) launch_reduce_multi(B, j, pass));
     CK(LC(p) launch_multiaxpy(B, SL_VBASE, j, SL_VJ1, pass));
   }
-  CK(LC(p) launch_dot(B, SL_VJ1, SL_VJ1));
   CK(LC(p) launch_reduce(B, B.off_vec, 1, 0, SS_GMRES_ARNOLDI, c.tol, j, c.restart));
   CK(LC(p) launch_axpby(B, AX_SCALE_INV_HNORM, SL_VJ1, SL_VJ1, -1));
   return PCB_OK;
@@ -1012,6 +1011,7 @@ static int fgmres_single(pcb_problem* p, const SolveCfg& c, int s_b, int s_x, Sc
       if (hs->flags & 8) break;
     }
     // x += Z y
+    CK(LC(p) launch_backsub(B));
     CK(LC(p) launch_multiaxpy(B, SL_ZBASE, k - 1, s_x, -1));
     CK(cudaMemsetAsync(&p->dSc->flags, 0, sizeof(int), p->stream));
     *it_out = total;
@@ -1738,9 +1738,7 @@ int round_step(BGroup& G, const SolveCfg& c) {
   } else {
     const int j = G.j;
     auto step = [&](const Batch& Bx) -> int {
-      CK(launch_setslot(Bx, SL_VJ, SL_VBASE, j));
-      CK(launch_setslot(Bx, SL_ZJ, SL_ZBASE, j));
-      CK(launch_setslot(Bx, SL_VJ1, SL_VBASE, j + 1));
+      CK(launch_setslots(Bx, SL_VJ, SL_ZJ, SL_VJ1, SL_VBASE, SL_ZBASE, j));
       int r;
       if ((r = apply_precond(p0, Bx, G.kind, G.prec, SL_VJ, SL_ZJ))) return r;
       CK(launch_matvec(Bx, G.op, SL_ZJ, SL_VJ1, -1, EPI_PLAIN));
@@ -1749,7 +1747,6 @@ int round_step(BGroup& G, const SolveCfg& c) {
         CK(launch_reduce_multi(Bx, j, pass));
         CK(launch_multiaxpy(Bx, SL_VBASE, j, SL_VJ1, pass));
       }
-      CK(launch_dot(Bx, SL_VJ1, SL_VJ1));
       CK(launch_reduce(Bx, Bx.off_vec, 1, 0, SS_GMRES_ARNOLDI, c.tol, j, c.restart));
       CK(launch_axpby(Bx, AX_SCALE_INV_HNORM, SL_VJ1, SL_VJ1, -1));
       return PCB_OK;
@@ -1776,6 +1773,7 @@ int round_step(BGroup& G, const SolveCfg& c) {
       std::vector<int> m2(n, 0);
       for (int k = 0; k < n; ++k) m2[k] = ending[k] && !G.done[k];
       if ((rc = set_active(G, m2))) return rc;
+      CK(launch_backsub(G.B));
       CK(launch_multiaxpy(G.B, SL_ZBASE, j, SL_XI, -1));
     }
     G.j += 1;
@@ -2145,7 +2143,7 @@ int srv_group_step(pcb_server* S, SrvGroup& G) {
       CK(launch_reduce(G.B, G.B.off_vec, 1, 0, SS_BNORM, tol, 0, 0));
       CK(launch_dot(G.B, SL_BI, SL_BI));
       CK(launch_reduce(G.B, G.B.off_vec, 1, 0, SS_GMRES_START, tol, 0, 0));
-      CK(launch_setslot(G.B, SL_VJ, SL_VBASE, 0, 0));
+      CK(launch_setslot(G.B, SL_VJ, SL_VBASE, 0));
       CK(launch_axpby(G.B, AX_SCALE_INV_BETA, SL_BI, SL_VJ, -1));
     }
     if ((rc = srv_read(G, st))) return rc;
@@ -2204,10 +2202,9 @@ int srv_group_step(pcb_server* S, SrvGroup& G) {
       CK(launch_matvec(G.B, G.op, SL_ZJ, SL_VJ1, -1, EPI_PLAIN));
       for (int pass = 0; pass < 2; ++pass) {
         CK(launch_multidot(G.B, SL_VBASE, -1, SL_VJ1, jmax));
-        CK(launch_reduce_multi(G.B, -1, pass));
+        CK(launch_reduce_multi(G.B, -1, pass, jmax));
         CK(launch_multiaxpy(G.B, SL_VBASE, -1, SL_VJ1, pass, jmax));
       }
-      CK(launch_dot(G.B, SL_VJ1, SL_VJ1));
       CK(launch_reduce(G.B, G.B.off_vec, 1, 0, SS_GMRES_ARNOLDI, tol, -1, restart));
       CK(launch_axpby(G.B, AX_SCALE_INV_HNORM, SL_VJ1, SL_VJ1, -1));
       if ((rc = srv_read(G, st))) return rc;
@@ -2227,6 +2224,7 @@ int srv_group_step(pcb_server* S, SrvGroup& G) {
           if (ending[k]) jend = std::max(jend, G.hSc[k].j - 1);
         }
         CK(cudaMemcpyAsync(G.dAct, G.hAct, sizeof(int) * G.cap, cudaMemcpyHostToDevice, st));
+        CK(launch_backsub(G.B));
         CK(launch_multiaxpy(G.B, SL_ZBASE, -1, SL_XI, -1, jend));
         for (int k = 0; k < G.cap; ++k) if (ending[k]) G.slots[k].phase = PH_END;
       }
