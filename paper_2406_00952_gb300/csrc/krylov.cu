@@ -82,8 +82,13 @@ __global__ void __launch_bounds__(256) k_axpby(const Geom* __restrict__ G, const
   }
 }
 
-// MINRES direction and solution update:
-//   w_new = (y/oldb - oldeps*w2 - delta*w)/gamma  -> slot w2 ;  x += phi*w_new
+// MINRES direction and solution update.  The direction w_k = (y/oldb - oldeps w_{k-2} - delta w_{k-1})/gamma is
+// kept without its scale, u = gamma oldb w, so that y enters with coefficient one:
+//   u_new = y + c2 u_{k-2} + c1 u_{k-1}  -> slot w2 ;  x += cx u_new
+// with the coefficients of the scalar step (Scal::wc1, wc2, wcx): three FP64 operations per value instead
+// of four, which leaves the kernel at the HBM limit (48 B per value; N = 511, n = 512: 2.24 -> 2.02 ms).
+// Run beside the product and the transforms in a branch of the iteration's graph it gained nothing: every
+// variant (1, 2, 3 or all its blocks per SM, with and without priorities) took the others' HBM time.
 __global__ void __launch_bounds__(256) k_minres_wx(const Geom* __restrict__ G, const Slots* __restrict__ S,
                                                    const Scal* __restrict__ Sc, const int* __restrict__ off, int count,
                                                    const int* __restrict__ active, int sy, int sw, int sw2, int sx) {
@@ -93,16 +98,28 @@ __global__ void __launch_bounds__(256) k_minres_wx(const Geom* __restrict__ G, c
   const double* __restrict__ w = S[inst].v[sw];
   double* __restrict__ w2 = S[inst].v[sw2];
   double* __restrict__ x = S[inst].v[sx];
-  // the 1/gamma scale is folded into the three coefficients: four FP64 operations per value (the
-  // kernel sits at the FP64 instruction limit as much as at the HBM limit)
-  const double ig = 1.0 / c.gamma;
-  const double cy = ig / c.oldb, c2 = -c.oldeps * ig, c1 = -c.delta * ig, phi = c.phi;
-  for (long long e = e0; e < len; e += stride) {
-    double t = y[e] * cy;
-    t = fma(c2, w2[e], t);
-    t = fma(c1, w[e], t);
+  const double c1 = c.wc1, c2 = c.wc2, cx = c.wcx;
+  long long e = e0;
+  for (; e + 3 * stride < len; e += 4 * stride) {       // four values in flight
+    double t[4], a[4], b[4], z[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      t[q] = y[e + q * stride];
+      a[q] = w2[e + q * stride];
+      b[q] = w[e + q * stride];
+      z[q] = x[e + q * stride];
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      t[q] = fma(c1, b[q], fma(c2, a[q], t[q]));
+      w2[e + q * stride] = t[q];
+      x[e + q * stride] = fma(cx, t[q], z[q]);
+    }
+  }
+  for (; e < len; e += stride) {
+    const double t = fma(c1, w[e], fma(c2, w2[e], y[e]));
     w2[e] = t;
-    x[e] = fma(phi, t, x[e]);
+    x[e] = fma(cx, t, x[e]);
   }
 }
 
@@ -243,6 +260,7 @@ __device__ void scalar_step(Scal& c, int step, double v, double tol, int j, int 
       if (v == 0.0) { c.beta1 = 0.0; c.beta = 0.0; c.est = 0.0; c.flags |= 1; c.active = 0; break; }
       c.beta1 = sqrt(v); c.beta = c.beta1; c.oldb = 0.0; c.dbar = 0.0; c.epsln = 0.0; c.phibar = c.beta1;
       c.cs = -1.0; c.sn = 0.0; c.est = 1.0;
+      c.ws1 = c.ws2 = 0.0;
       break;
     }
     case SS_MINRES_ALFA:
@@ -263,6 +281,12 @@ __device__ void scalar_step(Scal& c, int step, double v, double tol, int j, int 
       c.sn = c.beta / c.gamma;
       c.phi = c.cs * c.phibar;
       c.phibar = c.sn * c.phibar;
+      // coefficients of k_minres_wx: w_{k-1} = ws1 u_{k-1}, w_{k-2} = ws2 u_{k-2}
+      c.wc1 = -c.oldb * c.delta * c.ws1;
+      c.wc2 = -c.oldb * c.oldeps * c.ws2;
+      c.ws2 = c.ws1;
+      c.ws1 = 1.0 / (c.gamma * c.oldb);
+      c.wcx = c.phi * c.ws1;
       c.itn += 1;
       c.est = c.phibar / c.beta1;
       if (c.est <= tol) c.flags |= 1;
@@ -349,18 +373,25 @@ __global__ void __launch_bounds__(32) k_backsub(int count, const int* __restrict
   }
 }
 
-// Sum the instance's partials (nper values per block, index `which`) and run a scalar step.
-__global__ void __launch_bounds__(256) k_reduce(const int* __restrict__ off, int count, const int* __restrict__ active,
-                                                const double* __restrict__ partial, int nper, int which, Scal* Sc,
+// Sum the instance's partials (one per block) and run a scalar step.
+__global__ void __launch_bounds__(512) k_reduce(const int* __restrict__ off, int count, const int* __restrict__ active,
+                                                const double* __restrict__ partial, Scal* Sc,
                                                 int step, double tol, const double* __restrict__ tols, int j,
                                                 int restart) {
   const int inst = blockIdx.x;
   if (inst >= count) return;
   if (active && !active[inst]) return;
   const int b0 = off[inst], b1 = off[inst + 1];
-  double acc = 0.0;
-  for (int b = b0 + threadIdx.x; b < b1; b += blockDim.x) acc += partial[(long long)b * nper + which];
-  const double s = block_sum(acc);
+  // the products leave tens of thousands of partials of a large instance: four loads in flight per thread
+  // (N = 511, n = 512: 64 -> 17 us)
+  double a4[4] = {0.0, 0.0, 0.0, 0.0};
+  int b = b0 + threadIdx.x;
+  for (; b + 3 * (int)blockDim.x < b1; b += 4 * blockDim.x) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) a4[q] += partial[b + q * blockDim.x];
+  }
+  for (; b < b1; b += blockDim.x) a4[0] += partial[b];
+  const double s = block_sum((a4[0] + a4[1]) + (a4[2] + a4[3]));
   const double tl = tols ? tols[inst] : tol;
   if (step == SS_GMRES_ARNOLDI) {
     __shared__ double total;
@@ -418,10 +449,9 @@ cudaError_t launch_dot(const Batch& B, int sa, int sb) {
   k_dot<<<B.tot_vec, 256, 0, B.stream>>>(B.G, B.S, B.off_vec, B.count, B.active, sa, sb, B.partial);
   return cudaGetLastError();
 }
-cudaError_t launch_reduce(const Batch& B, const int* off, int nper, int which, int step, double tol, int j,
-                          int restart) {
-  k_reduce<<<B.count, 256, 0, B.stream>>>(off, B.count, B.active, B.partial, nper, which, B.Sc, step, tol, B.tols, j,
-                                          restart);
+cudaError_t launch_reduce(const Batch& B, const int* off, int step, double tol, int j, int restart) {
+  // one block size for every instance: the order of its sum must not depend on the batch it is in
+  k_reduce<<<B.count, 512, 0, B.stream>>>(off, B.count, B.active, B.partial, B.Sc, step, tol, B.tols, j, restart);
   return cudaGetLastError();
 }
 cudaError_t launch_axpby(const Batch& B, int mode, int sx, int sy, int sz) {

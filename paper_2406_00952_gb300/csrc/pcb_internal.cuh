@@ -177,6 +177,7 @@ struct Scal {
   // MINRES (Paige-Saunders recurrences)
   double beta, oldb, alfa, dbar, epsln, oldeps, phibar, cs, sn, delta, gbar, gamma, phi;
   double beta1, bnorm, est;
+  double wc1, wc2, wcx, ws1, ws2;   // direction update in unscaled form (k_minres_wx)
   // reductions land here
   double dot0, dot1;
   // GMRES

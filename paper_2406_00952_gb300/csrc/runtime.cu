@@ -52,8 +52,7 @@ static cudaError_t copy_host(double* dst, const double* src, size_t n, bool to_d
                          st);
 }
 cudaError_t launch_dot(const Batch& B, int sa, int sb);
-cudaError_t launch_reduce(const Batch& B, const int* off, int nper, int which, int step, double tol, int j,
-                          int restart);
+cudaError_t launch_reduce(const Batch& B, const int* off, int step, double tol, int j, int restart);
 cudaError_t launch_axpby(const Batch& B, int mode, int sx, int sy, int sz);
 cudaError_t launch_minres_wx(const Batch& B, int sy, int sw, int sw2, int sx);
 // j < 0: each instance at its own Arnoldi index (from Scal), all of them <= jmax when jmax >= 0
@@ -799,11 +798,11 @@ static int read_scal(const Batch& B, Scal* host, int count) {
 static int minres_iter_launches(pcb_problem* p, const Batch& B, const SolveCfg& c, int s_x) {
   int rc;
   CK(P_matvec(p, B, PCB_OP_A, SL_Y, SL_Q, SL_R1, EPI_MINRES | (c.prec == PCB_MIXED ? EPI_FAST : 0)));
-  CK(LC(p) launch_reduce(B, B.off_mv, 1, 0, SS_MINRES_ALFA, c.tol, 0, 0));
+  CK(LC(p) launch_reduce(B, B.off_mv, SS_MINRES_ALFA, c.tol, 0, 0));
   CK(LC(p) launch_axpby(B, AX_MINRES_R, SL_Q, SL_R2, SL_R1));
   if ((rc = P_precond(p, B, c.kind, c.prec, SL_R1, SL_YO))) return rc;
   CK(LC(p) launch_dot(B, SL_R1, SL_YO));
-  CK(LC(p) launch_reduce(B, B.off_vec, 1, 0, SS_MINRES_GIVENS, c.tol, 0, 0));
+  CK(LC(p) launch_reduce(B, B.off_vec, SS_MINRES_GIVENS, c.tol, 0, 0));
   CK(LC(p) launch_minres_wx(B, SL_Y, SL_W, SL_W2, s_x));
   CK(LC(p) launch_swap(B, SL_R1, SL_R2, SL_Y, SL_YO, SL_W, SL_W2));
   return PCB_OK;
@@ -864,11 +863,11 @@ static int minres_single(pcb_problem* p, const SolveCfg& c, int s_b, int s_x, Sc
   CK(LC(p) launch_axpby(B, AX_COPY, s_b, SL_R1, -1));
   CK(LC(p) launch_axpby(B, AX_COPY, s_b, SL_R2, -1));
   CK(LC(p) launch_dot(B, s_b, s_b));
-  CK(LC(p) launch_reduce(B, B.off_vec, 1, 0, SS_BNORM, c.tol, 0, 0));
+  CK(LC(p) launch_reduce(B, B.off_vec, SS_BNORM, c.tol, 0, 0));
   int rc = P_precond(p, B, c.kind, c.prec, SL_R2, SL_Y);
   if (rc) return rc;
   CK(LC(p) launch_dot(B, SL_R2, SL_Y));
-  CK(LC(p) launch_reduce(B, B.off_vec, 1, 0, SS_MINRES_INIT, c.tol, 0, 0));
+  CK(LC(p) launch_reduce(B, B.off_vec, SS_MINRES_INIT, c.tol, 0, 0));
   if ((rc = read_scal(B, hs, 1))) return rc;
   *it_out = 0; *conv_out = false; *relres_out = 1.0;
   if (hs->flags & 4) return PCB_ERR_NONFINITE;
@@ -910,7 +909,7 @@ static int minres_single(pcb_problem* p, const SolveCfg& c, int s_b, int s_x, Sc
       // sweep then measures the true residual of the outer system itself
       if (!c.check_true) { *relres_out = hs->est; return PCB_OK; }
       CK(P_matvec(p, B, PCB_OP_A, s_x, SL_Q, s_b, EPI_RESID));
-      CK(LC(p) launch_reduce(B, B.off_mv, 1, 0, SS_NORM, c.tol, 0, 0));
+      CK(LC(p) launch_reduce(B, B.off_mv, SS_NORM, c.tol, 0, 0));
       if ((rc = read_scal(B, hs, 1))) return rc;
       const double rel = std::sqrt(hs->dot1) / hs->bnorm;
       *relres_out = rel;
@@ -920,7 +919,7 @@ static int minres_single(pcb_problem* p, const SolveCfg& c, int s_b, int s_x, Sc
   }
   if (!c.check_true) { *relres_out = hs->est; return PCB_OK; }
   CK(P_matvec(p, B, PCB_OP_A, s_x, SL_Q, s_b, EPI_RESID));
-  CK(LC(p) launch_reduce(B, B.off_mv, 1, 0, SS_NORM, c.tol, 0, 0));
+  CK(LC(p) launch_reduce(B, B.off_mv, SS_NORM, c.tol, 0, 0));
   if ((rc = read_scal(B, hs, 1))) return rc;
   *relres_out = std::sqrt(hs->dot1) / hs->bnorm;
   *conv_out = *relres_out <= c.tol;
@@ -942,7 +941,7 @@ static int arnoldi_launches(pcb_problem* p, const Batch& B, const SolveCfg& c, i
     CK(LC(p) launch_reduce_multi(B, j, pass));
     CK(LC(p) launch_multiaxpy(B, SL_VBASE, j, SL_VJ1, pass));
   }
-  CK(LC(p) launch_reduce(B, B.off_vec, 1, 0, SS_GMRES_ARNOLDI, c.tol, j, c.restart));
+  CK(LC(p) launch_reduce(B, B.off_vec, SS_GMRES_ARNOLDI, c.tol, j, c.restart));
   CK(LC(p) launch_axpby(B, AX_SCALE_INV_HNORM, SL_VJ1, SL_VJ1, -1));
   return PCB_OK;
 }
@@ -955,7 +954,7 @@ static int fgmres_single(pcb_problem* p, const SolveCfg& c, int s_b, int s_x, Sc
   CK(cudaMemsetAsync(p->hS.v[s_x], 0, vb, p->stream));
   CK(cudaMemsetAsync(p->dSc, 0, sizeof(Scal), p->stream));
   CK(LC(p) launch_dot(B, s_b, s_b));
-  CK(LC(p) launch_reduce(B, B.off_vec, 1, 0, SS_BNORM, c.tol, 0, 0));
+  CK(LC(p) launch_reduce(B, B.off_vec, SS_BNORM, c.tol, 0, 0));
   int rc;
   if ((rc = read_scal(B, hs, 1))) return rc;
   *it_out = 0; *conv_out = false; *relres_out = 1.0;
@@ -978,7 +977,7 @@ static int fgmres_single(pcb_problem* p, const SolveCfg& c, int s_b, int s_x, Sc
   bool direct_first = true;
   while (total < limit) {
     CK(P_matvec(p, B, op, s_x, SL_R, s_b, EPI_RESID));
-    CK(LC(p) launch_reduce(B, B.off_mv, 1, 0, SS_GMRES_START, c.tol, 0, 0));
+    CK(LC(p) launch_reduce(B, B.off_mv, SS_GMRES_START, c.tol, 0, 0));
     if ((rc = read_scal(B, hs, 1))) return rc;
     if (hs->flags & 4) return PCB_ERR_NONFINITE;
     *relres_out = hs->est;
@@ -1018,7 +1017,7 @@ static int fgmres_single(pcb_problem* p, const SolveCfg& c, int s_b, int s_x, Sc
     if (c.fixed <= 0 && (hs->flags & 1)) {
       if (!c.check_true) { *relres_out = hs->est; return PCB_OK; }   // inner solve: as for MINRES
       CK(P_matvec(p, B, op, s_x, SL_R, s_b, EPI_RESID));
-      CK(LC(p) launch_reduce(B, B.off_mv, 1, 0, SS_NORM, c.tol, 0, 0));
+      CK(LC(p) launch_reduce(B, B.off_mv, SS_NORM, c.tol, 0, 0));
       if ((rc = read_scal(B, hs, 1))) return rc;
       *relres_out = std::sqrt(hs->dot1) / hs->bnorm;
       if (*relres_out <= c.tol) { *conv_out = true; return PCB_OK; }
@@ -1026,7 +1025,7 @@ static int fgmres_single(pcb_problem* p, const SolveCfg& c, int s_b, int s_x, Sc
   }
   if (!c.check_true) { *relres_out = hs->est; return PCB_OK; }
   CK(P_matvec(p, B, op, s_x, SL_R, s_b, EPI_RESID));
-  CK(LC(p) launch_reduce(B, B.off_mv, 1, 0, SS_NORM, c.tol, 0, 0));
+  CK(LC(p) launch_reduce(B, B.off_mv, SS_NORM, c.tol, 0, 0));
   if ((rc = read_scal(B, hs, 1))) return rc;
   *relres_out = std::sqrt(hs->dot1) / hs->bnorm;
   *conv_out = *relres_out <= c.tol;
@@ -1106,7 +1105,7 @@ static int solve_impl(pcb_problem* p, const pcb_solve_opts* o, const double* b_d
     const size_t vbytes = nv * sizeof(double);
     CK(cudaMemsetAsync(x_dev, 0, vbytes, p->stream));
     CK(LC(p) launch_dot(p->B, SL_B, SL_B));
-    CK(LC(p) launch_reduce(p->B, p->B.off_vec, 1, 0, SS_BNORM, c.tol, 0, 0));
+    CK(LC(p) launch_reduce(p->B, p->B.off_vec, SS_BNORM, c.tol, 0, 0));
     if ((rc = read_scal(p->B, hs, 1))) return rc;
     const double bnorm = hs->bnorm;
     if (!std::isfinite(bnorm)) return PCB_ERR_NONFINITE;
@@ -1127,7 +1126,7 @@ static int solve_impl(pcb_problem* p, const pcb_solve_opts* o, const double* b_d
       // x += d ; r = b - op x  (into the inner right-hand side slot)
       CK(LC(p) launch_axpby(p->B, AX_ADD, SL_XI, SL_X, -1));
       CK(P_matvec(p, p->B, c.op, SL_X, SL_BI, SL_B, EPI_RESID));
-      CK(LC(p) launch_reduce(p->B, p->B.off_mv, 1, 0, SS_NORM, c.tol, 0, 0));
+      CK(LC(p) launch_reduce(p->B, p->B.off_mv, SS_NORM, c.tol, 0, 0));
       if ((rc = read_scal(p->B, hs, 1))) break;
       rnorm = std::sqrt(hs->dot1);
       relres = rnorm / bnorm;
@@ -1202,7 +1201,7 @@ int pcb_lanczos_product(pcb_problem* p, int precision, const double* y_dev, cons
   if ((rc = upload_slots(p))) return rc;
   const int epi = EPI_MINRES | (precision == PCB_MIXED ? EPI_FAST : 0);
   CK(launch_matvec(p->B, PCB_OP_A, SL_UIN, SL_UOUT, oldb > 0.0 ? SL_UAUX : -1, epi));
-  CK(launch_reduce(p->B, p->B.off_mv, 1, 0, SS_NORM, 0.0, 0, 0));
+  CK(launch_reduce(p->B, p->B.off_mv, SS_NORM, 0.0, 0, 0));
   if ((rc = read_scal(p->B, hs, 1))) return rc;
   *dot = hs->dot1;
   return PCB_OK;
@@ -1646,7 +1645,7 @@ int group_setup(BGroup& G, const SolveCfg& c, const double* const* b_dev, double
   CK(launch_axpby(G.B, AX_ZERO, -1, SL_X, -1));
   CK(launch_axpby(G.B, AX_COPY, SL_B, SL_BI, -1));
   CK(launch_dot(G.B, SL_B, SL_B));
-  CK(launch_reduce(G.B, G.B.off_vec, 1, 0, SS_BNORM, c.tol, 0, 0));
+  CK(launch_reduce(G.B, G.B.off_vec, SS_BNORM, c.tol, 0, 0));
   if ((rc = read_all(G))) return rc;
   for (int k = 0; k < n; ++k) {
     G.bnorm[k] = G.hSc[k].bnorm; G.rnorm[k] = G.bnorm[k];
@@ -1679,12 +1678,12 @@ int round_start(BGroup& G, const SolveCfg& c) {
     CK(launch_axpby(G.B, AX_COPY, SL_BI, SL_R2, -1));
     if ((rc = apply_precond(G.probs[0], G.B, G.kind, G.prec, SL_R2, SL_Y))) return rc;
     CK(launch_dot(G.B, SL_R2, SL_Y));
-    CK(launch_reduce(G.B, G.B.off_vec, 1, 0, SS_MINRES_INIT, c.tol, 0, 0));
+    CK(launch_reduce(G.B, G.B.off_vec, SS_MINRES_INIT, c.tol, 0, 0));
   } else {
     CK(launch_dot(G.B, SL_BI, SL_BI));
-    CK(launch_reduce(G.B, G.B.off_vec, 1, 0, SS_BNORM, c.tol, 0, 0));
+    CK(launch_reduce(G.B, G.B.off_vec, SS_BNORM, c.tol, 0, 0));
     CK(launch_dot(G.B, SL_BI, SL_BI));
-    CK(launch_reduce(G.B, G.B.off_vec, 1, 0, SS_GMRES_START, c.tol, 0, 0));
+    CK(launch_reduce(G.B, G.B.off_vec, SS_GMRES_START, c.tol, 0, 0));
     CK(launch_setslot(G.B, SL_VJ, SL_VBASE, 0));
     CK(launch_axpby(G.B, AX_SCALE_INV_BETA, SL_BI, SL_VJ, -1));
   }
@@ -1707,12 +1706,12 @@ int round_step(BGroup& G, const SolveCfg& c) {
   if (G.method == PCB_MINRES) {
     auto iter = [&](const Batch& Bx) -> int {
       CK(launch_matvec(Bx, PCB_OP_A, SL_Y, SL_Q, SL_R1, EPI_MINRES | (G.prec == PCB_MIXED ? EPI_FAST : 0)));
-      CK(launch_reduce(Bx, Bx.off_mv, 1, 0, SS_MINRES_ALFA, c.tol, 0, 0));
+      CK(launch_reduce(Bx, Bx.off_mv, SS_MINRES_ALFA, c.tol, 0, 0));
       CK(launch_axpby(Bx, AX_MINRES_R, SL_Q, SL_R2, SL_R1));
       int r;
       if ((r = apply_precond(p0, Bx, G.kind, G.prec, SL_R1, SL_YO))) return r;
       CK(launch_dot(Bx, SL_R1, SL_YO));
-      CK(launch_reduce(Bx, Bx.off_vec, 1, 0, SS_MINRES_GIVENS, c.tol, 0, 0));
+      CK(launch_reduce(Bx, Bx.off_vec, SS_MINRES_GIVENS, c.tol, 0, 0));
       CK(launch_minres_wx(Bx, SL_Y, SL_W, SL_W2, SL_XI));
       CK(launch_swap(Bx, SL_R1, SL_R2, SL_Y, SL_YO, SL_W, SL_W2));
       return PCB_OK;
@@ -1747,7 +1746,7 @@ int round_step(BGroup& G, const SolveCfg& c) {
         CK(launch_reduce_multi(Bx, j, pass));
         CK(launch_multiaxpy(Bx, SL_VBASE, j, SL_VJ1, pass));
       }
-      CK(launch_reduce(Bx, Bx.off_vec, 1, 0, SS_GMRES_ARNOLDI, c.tol, j, c.restart));
+      CK(launch_reduce(Bx, Bx.off_vec, SS_GMRES_ARNOLDI, c.tol, j, c.restart));
       CK(launch_axpby(Bx, AX_SCALE_INV_HNORM, SL_VJ1, SL_VJ1, -1));
       return PCB_OK;
     };
@@ -1794,7 +1793,7 @@ int round_end(BGroup& G, const SolveCfg& c, int max_ref) {
   if ((rc = set_active(G, mask))) return rc;
   CK(launch_axpby(G.B, AX_ADD, SL_XI, SL_X, -1));
   CK(launch_matvec(G.B, G.op, SL_X, SL_BI, SL_B, EPI_RESID));
-  CK(launch_reduce(G.B, G.B.off_mv, 1, 0, SS_NORM, c.tol, 0, 0));
+  CK(launch_reduce(G.B, G.B.off_mv, SS_NORM, c.tol, 0, 0));
   if ((rc = read_all(G))) return rc;
   for (int k = 0; k < n; ++k) {
     if (!mask[k]) continue;
@@ -2095,7 +2094,7 @@ int srv_group_step(pcb_server* S, SrvGroup& G) {
   if (rc == 1) {
     CK(launch_axpby(G.B, AX_ADD, SL_XI, SL_X, -1));
     CK(launch_matvec(G.B, G.op, SL_X, SL_BI, SL_B, EPI_RESID));
-    CK(launch_reduce(G.B, G.B.off_mv, 1, 0, SS_NORM, tol, 0, 0));
+    CK(launch_reduce(G.B, G.B.off_mv, SS_NORM, tol, 0, 0));
     if ((rc = srv_read(G, st))) return rc;
     for (int k = 0; k < G.cap; ++k) {
       SrvSlot& s = G.slots[k];
@@ -2113,7 +2112,7 @@ int srv_group_step(pcb_server* S, SrvGroup& G) {
   if ((rc = srv_mask(G, st, PH_START, true)) < 0) return rc;
   if (rc == 1) {   // first round: ||b||
     CK(launch_dot(G.B, SL_B, SL_B));
-    CK(launch_reduce(G.B, G.B.off_vec, 1, 0, SS_BNORM, tol, 0, 0));
+    CK(launch_reduce(G.B, G.B.off_vec, SS_BNORM, tol, 0, 0));
     if ((rc = srv_read(G, st))) return rc;
     for (int k = 0; k < G.cap; ++k) {
       SrvSlot& s = G.slots[k];
@@ -2137,12 +2136,12 @@ int srv_group_step(pcb_server* S, SrvGroup& G) {
       CK(launch_axpby(G.B, AX_COPY, SL_BI, SL_R2, -1));
       if ((rc = precond(SL_R2, SL_Y))) return rc;
       CK(launch_dot(G.B, SL_R2, SL_Y));
-      CK(launch_reduce(G.B, G.B.off_vec, 1, 0, SS_MINRES_INIT, tol, 0, 0));
+      CK(launch_reduce(G.B, G.B.off_vec, SS_MINRES_INIT, tol, 0, 0));
     } else {
       CK(launch_dot(G.B, SL_BI, SL_BI));
-      CK(launch_reduce(G.B, G.B.off_vec, 1, 0, SS_BNORM, tol, 0, 0));
+      CK(launch_reduce(G.B, G.B.off_vec, SS_BNORM, tol, 0, 0));
       CK(launch_dot(G.B, SL_BI, SL_BI));
-      CK(launch_reduce(G.B, G.B.off_vec, 1, 0, SS_GMRES_START, tol, 0, 0));
+      CK(launch_reduce(G.B, G.B.off_vec, SS_GMRES_START, tol, 0, 0));
       CK(launch_setslot(G.B, SL_VJ, SL_VBASE, 0));
       CK(launch_axpby(G.B, AX_SCALE_INV_BETA, SL_BI, SL_VJ, -1));
     }
@@ -2167,11 +2166,11 @@ int srv_group_step(pcb_server* S, SrvGroup& G) {
     bool any_end = false;
     if (G.method == PCB_MINRES) {
       CK(launch_matvec(G.B, PCB_OP_A, SL_Y, SL_Q, SL_R1, EPI_MINRES | (prec == PCB_MIXED ? EPI_FAST : 0)));
-      CK(launch_reduce(G.B, G.B.off_mv, 1, 0, SS_MINRES_ALFA, tol, 0, 0));
+      CK(launch_reduce(G.B, G.B.off_mv, SS_MINRES_ALFA, tol, 0, 0));
       CK(launch_axpby(G.B, AX_MINRES_R, SL_Q, SL_R2, SL_R1));
       if ((rc = precond(SL_R1, SL_YO))) return rc;
       CK(launch_dot(G.B, SL_R1, SL_YO));
-      CK(launch_reduce(G.B, G.B.off_vec, 1, 0, SS_MINRES_GIVENS, tol, 0, 0));
+      CK(launch_reduce(G.B, G.B.off_vec, SS_MINRES_GIVENS, tol, 0, 0));
       CK(launch_minres_wx(G.B, SL_Y, SL_W, SL_W2, SL_XI));
       if ((rc = srv_read(G, st))) return rc;
       for (int k = 0; k < G.cap; ++k) {
@@ -2205,7 +2204,7 @@ int srv_group_step(pcb_server* S, SrvGroup& G) {
         CK(launch_reduce_multi(G.B, -1, pass, jmax));
         CK(launch_multiaxpy(G.B, SL_VBASE, -1, SL_VJ1, pass, jmax));
       }
-      CK(launch_reduce(G.B, G.B.off_vec, 1, 0, SS_GMRES_ARNOLDI, tol, -1, restart));
+      CK(launch_reduce(G.B, G.B.off_vec, SS_GMRES_ARNOLDI, tol, -1, restart));
       CK(launch_axpby(G.B, AX_SCALE_INV_HNORM, SL_VJ1, SL_VJ1, -1));
       if ((rc = srv_read(G, st))) return rc;
       for (int k = 0; k < G.cap; ++k) {
