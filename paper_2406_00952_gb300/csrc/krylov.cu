@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(256) k_axpby(const Geom* __restrict__ G, const
   } else if (mode == AX_MINRES_R) {
     // z = x - (alfa/beta) y  written to slot sz  (x = q, y = r2, z = r1 slot)
     double* __restrict__ z = S[inst].v[sz];
-    const double f = -c.alfa / c.beta;
+    const double f = c.rf;
     for (long long e = e0; e < len; e += stride) z[e] = fma(f, y[e], x[e]);
   } else if (mode == AX_SCALE_INV_BETA) {
     const double f = 1.0 / c.beta;
@@ -265,6 +265,7 @@ __device__ void scalar_step(Scal& c, int step, double v, double tol, int j, int 
     }
     case SS_MINRES_ALFA:
       c.alfa = v;
+      c.rf = -v / c.beta;
       break;
     case SS_MINRES_GIVENS: {
       c.oldb = c.beta;

@@ -177,6 +177,7 @@ struct Scal {
   // MINRES (Paige-Saunders recurrences)
   double beta, oldb, alfa, dbar, epsln, oldeps, phibar, cs, sn, delta, gbar, gamma, phi;
   double beta1, bnorm, est;
+  double rf;                        // -alfa/beta: residual update r1 = q + rf r2
   double wc1, wc2, wcx, ws1, ws2;   // direction update in unscaled form (k_minres_wx)
   // reductions land here
   double dot0, dot1;
@@ -293,6 +294,7 @@ struct Batch {
   const int* lane_sp[2];
   const int* lane_tm[2];
   unsigned lane_sp_set[2], lane_tm_set[2];
+  int fuse_r2, fuse_z;    // vector slots of the fused passes (launch_precond_minres)
   int t512v;              // 1 / 2: the n = 512 time pass runs its three / four-blocks-per-SM variant
                           // (every instance of the batch that takes that pass chose it)
   int fem_m;              // > 0: a single finite-element instance with m = fem_m spatial points

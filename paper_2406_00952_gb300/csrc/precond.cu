@@ -877,6 +877,19 @@ cudaError_t launch_fem_spatial(const Batch& B, int mode, int op, int in_slot, in
   return dst_pass<double>(B, 5, -1, out_slot);
 }
 
+// MINRES's residual update, preconditioner and inner product in the five passes: r1 = q + rf r2 (scalars of
+// the instance) to slot r1, y = P^{-1} r1 to slot y, partial[b] = the blocks' sums of r1 . y over B.off_ls[1].
+// *fused = false, and nothing launched, unless every instance takes the one-line-per-lane FP32 passes on
+// a Dirichlet grid.  (B.fuse_z != 0 marks the fused passes: slot 0 is never a Krylov vector.)
+cudaError_t launch_precond_minres(const Batch& B, int kind, int prec, int q, int r2, int r1, int y, bool* fused) {
+  *fused = prec == PCB_MIXED && B.lane_sp_set[1] && B.tot_dst_i[1] == 0 && !(B.lane_sp_set[1] >> 12);
+  if (!*fused) return cudaSuccess;
+  Batch F = B;
+  F.fuse_r2 = r2;
+  F.fuse_z = r1;
+  return lane_passes<float>(F, kind, q, y);
+}
+
 // B.dst_q / B.time_q = 0 selects the shared-launch kernels for instances of different sizes.
 cudaError_t launch_precond_fast(const Batch& B, int kind, int prec, int in_slot, int out_slot) {
   return prec == PCB_MIXED ? precond_passes<float>(B, kind, in_slot, out_slot)

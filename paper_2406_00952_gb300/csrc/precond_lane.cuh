@@ -120,6 +120,13 @@ template <> struct Pairs<double> {
   __device__ __forceinline__ void put(int at, double2 v) const { p[at] = v.x; q[at] = v.y; }
 };
 
+// What a pass of a MINRES iteration takes over from the vector kernels around the apply (see FUSE)
+struct LaneFuse {
+  const Scal* Sc;
+  double* partial;
+  int r2, z;
+};
+
 // Bring a line towards L2.  A block asks for the tile `ahead` blocks on, which starts about when it
 // ends: HBM then works through the register steps, and the loads of a tile find most of it in L2.
 // (N = 511, n = 512: pass 2 0.41 -> 0.39 ms, pass 4 0.42 -> 0.39.  Not for FP64 rows, which start at any
@@ -215,11 +222,14 @@ constexpr int spatial_blocks() {
 // registers and stores straight from them: LT adjacent columns are one contiguous segment.
 // USER: the input is a vector slot.  An FP32 pass converts it on its way to the exchange memory first:
 // 2 A FP64 values in registers would spill.
+// FUSE (FP32, USER): the input is MINRES's residual r1 = q + rf r2 (q = in_sel, rf = -alfa/beta from the
+// scalar step), formed here and written to slot fuse.z, instead of by a kernel of its own that this pass
+// would read again: 28 B a value in one launch instead of 24 + 12 (N = 511, n = 512: 0.94 + 0.61 -> 1.26 ms).
 // ------------------------------------------------------------------------------------------
-template <typename R, int M, bool EV, bool USER>
+template <typename R, int M, bool EV, bool USER, bool FUSE>
 __global__ void __launch_bounds__(spatial_threads<R, M>(), spatial_blocks<R, M>())
     k_lane_rows(const Geom* __restrict__ G, const Slots* __restrict__ S, const int* __restrict__ off, int count, Sel sel,
-                int in_sel, int out_sel, int inv, int ahead) {
+                int in_sel, int out_sel, int inv, LaneFuse fuse, int ahead) {
   using T = cx<R>;
   constexpr int A = Shape<M>::A, B = Shape<M>::B, NG = Shape<M>::GROUPS, LT = spatial_lanes<R, M>();
   constexpr bool STAGED = USER && sizeof(R) == 4;
@@ -247,8 +257,11 @@ __global__ void __launch_bounds__(spatial_threads<R, M>(), spatial_blocks<R, M>(
       // sends the thread through its rows once more.
       const double* __restrict__ in0 = (const double*)v.base + at0;
       const double* __restrict__ in1 = in0 + v.hs;
-      constexpr int U = M >= 1024 ? 16 : 8;
+      constexpr int U = FUSE ? (M >= 512 ? 8 : 4) : M >= 1024 ? 16 : 8;
       unsigned rare = 0;
+      const double rf = FUSE ? fuse.Sc[inst].rf : 0.0;
+      const double* __restrict__ r0 = FUSE ? S[inst].v[fuse.r2] + at0 : nullptr;
+      double* __restrict__ z0 = FUSE ? S[inst].v[fuse.z] + at0 : nullptr;
       for (int r = grp; r < N; r += U * NG) {
         double a[U], b[U];
 #pragma unroll
@@ -256,6 +269,24 @@ __global__ void __launch_bounds__(spatial_threads<R, M>(), spatial_blocks<R, M>(
           const int at = min(r + u * NG, N - 1) * rs;
           a[u] = in0[at];
           b[u] = in1[at];
+        }
+        if constexpr (FUSE) {
+          double c[U], d[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int at = min(r + u * NG, N - 1) * rs;
+            c[u] = r0[at];
+            d[u] = r0[v.hs + at];
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            a[u] = fma(rf, c[u], a[u]);
+            b[u] = fma(rf, d[u], b[u]);
+            if (ok && r + u * NG < N) {
+              z0[(r + u * NG) * rs] = a[u];
+              z0[v.hs + (r + u * NG) * rs] = b[u];
+            }
+          }
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -265,7 +296,14 @@ __global__ void __launch_bounds__(spatial_threads<R, M>(), spatial_blocks<R, M>(
       }
       if (rare) {
 #pragma unroll 1
-        for (int r = grp; r < N; r += NG) ex[r * LT] = mk<R>((R)in0[r * rs], (R)in1[r * rs]);
+        for (int r = grp; r < N; r += NG) {
+          double a = in0[r * rs], b = in1[r * rs];
+          if (FUSE) {
+            a = fma(rf, r0[r * rs], a);
+            b = fma(rf, r0[v.hs + r * rs], b);
+          }
+          ex[r * LT] = mk<R>((R)a, (R)b);
+        }
       }
       __syncthreads();
       if (first) gather<R, M, EV>(x, grp, inv != 0, [&](int at) { return ex[at * LT]; });
@@ -303,6 +341,9 @@ __global__ void __launch_bounds__(spatial_threads<R, M>(), spatial_blocks<R, M>(
 // a slice; value p of row r goes to out[p rs + r].  The rows come in with 8-byte asynchronous copies
 // (coalesced along the row) and are read back one line per lane (odd pitch); the exchange reuses that
 // memory.  USER: the output is a vector slot.
+// FUSE (FP32, USER): also leaves partial[block] = sum of the output times slot fuse.z over the tile, the
+// inner product r1 . y of MINRES, whose kernel would read the output again: 20 B a value instead of
+// 12 + 16 (N = 511, n = 512: 0.65 + 0.60 -> 1.07 ms).
 // ------------------------------------------------------------------------------------------
 template <int M, bool EV>
 constexpr int cols_pitch() { return (EV ? M / 2 + 1 : M / 2 - 1) | 1; }
@@ -312,10 +353,10 @@ constexpr size_t cols_smem() {
   return rows > spatial_smem<R, M>() ? rows : spatial_smem<R, M>();
 }
 
-template <typename R, int M, bool EV, bool USER>
+template <typename R, int M, bool EV, bool USER, bool FUSE>
 __global__ void __launch_bounds__(spatial_threads<R, M>(), spatial_blocks<R, M>())
     k_lane_cols(const Geom* __restrict__ G, const Slots* __restrict__ S, const int* __restrict__ off, int count, Sel sel,
-                int in_sel, int out_sel, int inv, int ahead) {
+                int in_sel, int out_sel, int inv, LaneFuse fuse, int ahead) {
   using T = cx<R>;
   constexpr int A = Shape<M>::A, B = Shape<M>::B, NG = Shape<M>::GROUPS, LT = spatial_lanes<R, M>();
   constexpr int N = EV ? M / 2 + 1 : M / 2 - 1, PITCH = cols_pitch<M, EV>(), NT = spatial_threads<R, M>();
@@ -399,27 +440,56 @@ __global__ void __launch_bounds__(spatial_threads<R, M>(), spatial_blocks<R, M>(
   if constexpr (STAGED) {
     // FP32 -> FP64 on the way out, as on the way in (k_lane_rows)
     __syncthreads();
-    if (!ok) return;
     double* __restrict__ out0 = (double*)v.base + at0;
     double* __restrict__ out1 = out0 + v.hs;
-    constexpr int U = 4;
+    const double* __restrict__ z0 = FUSE ? S[inst].v[fuse.z] + at0 : nullptr;
+    constexpr int U = FUSE && M >= 512 ? 8 : 4;
     const T* src = ex + (EV ? 0 : LT);
     unsigned rare = 0;
-    for (int p = grp; p < N; p += U * NG) {
+    double dot = 0.0;
+    if (ok)
+      for (int p = grp; p < N; p += U * NG) {
+        double za[U], zb[U];
+        if constexpr (FUSE) {
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (p + u * NG < N) {
-          const T z = src[(p + u * NG) * LT];
-          out0[(p + u * NG) * rs] = f2d_plain(z.x, rare);
-          out1[(p + u * NG) * rs] = f2d_plain(z.y, rare);
+          for (int u = 0; u < U; ++u) {
+            const int at = min(p + u * NG, N - 1) * rs;
+            za[u] = z0[at];
+            zb[u] = z0[v.hs + at];
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          if (p + u * NG < N) {
+            const T z = src[(p + u * NG) * LT];
+            const double a = f2d_plain(z.x, rare), b = f2d_plain(z.y, rare);
+            out0[(p + u * NG) * rs] = a;
+            out1[(p + u * NG) * rs] = b;
+            if constexpr (FUSE) dot = fma(b, zb[u], fma(a, za[u], dot));
+          }
         }
       }
-    }
-    if (rare) {
+    if (ok && rare) {
+      dot = 0.0;
 #pragma unroll 1
       for (int p = grp; p < N; p += NG) {
-        out0[p * rs] = (double)src[p * LT].x;
-        out1[p * rs] = (double)src[p * LT].y;
+        const double a = src[p * LT].x, b = src[p * LT].y;
+        out0[p * rs] = a;
+        out1[p * rs] = b;
+        if constexpr (FUSE) dot = fma(b, z0[v.hs + p * rs], fma(a, z0[p * rs], dot));
+      }
+    }
+    if constexpr (FUSE) {
+      // sixteen lanes at a time: the last warp of a block may be half a warp
+      __shared__ double red[NT / 16];
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) dot += __shfl_xor_sync(threadIdx.x & 16 ? 0xffff0000u : 0x0000ffffu, dot, o, 16);
+      if (threadIdx.x % 16 == 0) red[threadIdx.x / 16] = dot;
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        double sum = 0.0;
+        for (int k = 0; k < NT / 16; ++k) sum += red[k];
+        fuse.partial[blockIdx.x] = sum;
       }
     }
   }
@@ -743,19 +813,19 @@ cudaError_t launch(K kern, DeviceInt& resident, int blocks, int threads, size_t 
   return cudaGetLastError();
 }
 
-template <typename R, int M, bool EV, bool USER>
+template <typename R, int M, bool EV, bool USER, bool FUSE = false>
 cudaError_t rows_pass(const Batch& B, Sel sel, int in_sel, int out_sel, int inv) {
   constexpr int p = sizeof(R) == 4;
   static DeviceInt resident;
-  return launch(k_lane_rows<R, M, EV, USER>, resident, B.tot_ls[p], spatial_threads<R, M>(), spatial_smem<R, M>(),
-                B.stream, B.G, (const Slots*)B.S, B.off_ls[p], B.count, sel, in_sel, out_sel, inv);
+  return launch(k_lane_rows<R, M, EV, USER, FUSE>, resident, B.tot_ls[p], spatial_threads<R, M>(), spatial_smem<R, M>(),
+                B.stream, B.G, (const Slots*)B.S, B.off_ls[p], B.count, sel, in_sel, out_sel, inv, LaneFuse{B.Sc, B.partial, B.fuse_r2, B.fuse_z});
 }
-template <typename R, int M, bool EV, bool USER>
+template <typename R, int M, bool EV, bool USER, bool FUSE = false>
 cudaError_t cols_pass(const Batch& B, Sel sel, int in_sel, int out_sel, int inv) {
   constexpr int p = sizeof(R) == 4;
   static DeviceInt resident;
-  return launch(k_lane_cols<R, M, EV, USER>, resident, B.tot_ls[p], spatial_threads<R, M>(), cols_smem<R, M, EV>(),
-                B.stream, B.G, (const Slots*)B.S, B.off_ls[p], B.count, sel, in_sel, out_sel, inv);
+  return launch(k_lane_cols<R, M, EV, USER, FUSE>, resident, B.tot_ls[p], spatial_threads<R, M>(), cols_smem<R, M, EV>(),
+                B.stream, B.G, (const Slots*)B.S, B.off_ls[p], B.count, sel, in_sel, out_sel, inv, LaneFuse{B.Sc, B.partial, B.fuse_r2, B.fuse_z});
 }
 template <typename R, int n, bool GZ>
 cudaError_t time_pass_n(const Batch& B, Sel sel, int kind, int in_sel, int out_sel) {

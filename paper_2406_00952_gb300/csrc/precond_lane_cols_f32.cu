@@ -7,6 +7,8 @@ namespace {
 template <int M, bool EV>
 struct Cols {
   static cudaError_t run(const Batch& B, Sel sel, int stage, int in_sel, int out_sel) {
+    if constexpr (!EV)      // MINRES runs on Dirichlet grids
+      if (stage == 5 && B.fuse_z) return lane::cols_pass<float, M, false, true, true>(B, sel, in_sel, out_sel, 1);
     return stage == 2 ? lane::cols_pass<float, M, EV, false>(B, sel, in_sel, out_sel, 0)
                       : lane::cols_pass<float, M, EV, true>(B, sel, in_sel, out_sel, 1);
   }

@@ -7,6 +7,8 @@ namespace {
 template <int M, bool EV>
 struct Rows {
   static cudaError_t run(const Batch& B, Sel sel, int stage, int in_sel, int out_sel) {
+    if constexpr (!EV)      // MINRES runs on Dirichlet grids
+      if (stage == 1 && B.fuse_z) return lane::rows_pass<float, M, false, true, true>(B, sel, in_sel, out_sel, 0);
     return stage == 1 ? lane::rows_pass<float, M, EV, true>(B, sel, in_sel, out_sel, 0)
                       : lane::rows_pass<float, M, EV, false>(B, sel, in_sel, out_sel, 1);
   }

@@ -20,6 +20,7 @@
 namespace pcb {
 // launchers defined in the other translation units
 cudaError_t launch_precond_fast(const Batch& B, int kind, int prec, int in_slot, int out_slot);
+cudaError_t launch_precond_minres(const Batch& B, int kind, int prec, int q, int r2, int r1, int y, bool* fused);
 cudaError_t launch_precond_mg(const Batch& B, const Geom& g, int kind, int prec, int cycles, int in_slot,
                               int out_slot);
 void mg_release(const void* ws);
@@ -657,7 +658,7 @@ int pcb_create(const pcb_desc* d_in, pcb_problem** out) {
   if (cudaMalloc(&p->dG, sizeof(Geom)) != cudaSuccess || cudaMalloc(&p->dS, sizeof(Slots)) != cudaSuccess ||
       cudaMalloc(&p->dSc, sizeof(Scal)) != cudaSuccess || cudaMalloc(&p->doff, batch_ints(1) * sizeof(int)) != cudaSuccess ||
       cudaMalloc(&p->partial, (size_t)g.vec_blocks * (PCB_MAX_RESTART + 2) * sizeof(double) +
-                                  (size_t)std::max(g.mv_blocks, 1) * sizeof(double)) != cudaSuccess)
+                                  (size_t)std::max(std::max(g.mv_blocks, g.ls_blocks[1]), 1) * sizeof(double)) != cudaSuccess)
     return fail(PCB_ERR_OUT_OF_MEMORY);
   if (cudaMallocHost(&p->hSc, sizeof(Scal)) != cudaSuccess || cudaMallocHost(&p->hSpin, sizeof(Slots)) != cudaSuccess)
     return fail(PCB_ERR_OUT_OF_MEMORY);
@@ -799,10 +800,20 @@ static int minres_iter_launches(pcb_problem* p, const Batch& B, const SolveCfg& 
   int rc;
   CK(P_matvec(p, B, PCB_OP_A, SL_Y, SL_Q, SL_R1, EPI_MINRES | (c.prec == PCB_MIXED ? EPI_FAST : 0)));
   CK(LC(p) launch_reduce(B, B.off_mv, SS_MINRES_ALFA, c.tol, 0, 0));
-  CK(LC(p) launch_axpby(B, AX_MINRES_R, SL_Q, SL_R2, SL_R1));
-  if ((rc = P_precond(p, B, c.kind, c.prec, SL_R1, SL_YO))) return rc;
-  CK(LC(p) launch_dot(B, SL_R1, SL_YO));
-  CK(LC(p) launch_reduce(B, B.off_vec, SS_MINRES_GIVENS, c.tol, 0, 0));
+  // residual update, preconditioner and inner product: in the preconditioner's own passes where it can be
+  // (a profiled solve times the preconditioner, so it keeps them apart)
+  bool fused = false;
+  if (!p->prof && c.kind != PCB_PREC_NONE && !p->g.mg_route)
+    CK(launch_precond_minres(B, c.kind, c.prec, SL_Q, SL_R2, SL_R1, SL_YO, &fused));
+  if (fused) {
+    p->launches += precond_launch_count(false, c.kind);
+    p->prec_applies += 1;
+  } else {
+    CK(LC(p) launch_axpby(B, AX_MINRES_R, SL_Q, SL_R2, SL_R1));
+    if ((rc = P_precond(p, B, c.kind, c.prec, SL_R1, SL_YO))) return rc;
+    CK(LC(p) launch_dot(B, SL_R1, SL_YO));
+  }
+  CK(LC(p) launch_reduce(B, fused ? B.off_ls[1] : B.off_vec, SS_MINRES_GIVENS, c.tol, 0, 0));
   CK(LC(p) launch_minres_wx(B, SL_Y, SL_W, SL_W2, s_x));
   CK(LC(p) launch_swap(B, SL_R1, SL_R2, SL_Y, SL_YO, SL_W, SL_W2));
   return PCB_OK;
@@ -1617,9 +1628,9 @@ int group_setup(BGroup& G, const SolveCfg& c, const double* const* b_dev, double
     S.v[SL_B] = (double*)b_dev[G.idx[k]];
     gs.push_back(p->g);
   }
-  size_t part = 0; int tv = 0, tm = 0;
-  for (const Geom& g : gs) { tv += g.vec_blocks; tm += g.mv_blocks; }
-  part = std::max((size_t)tv * (PCB_MAX_RESTART + 1), (size_t)tm) + 1;
+  size_t part = 0; int tv = 0, tm = 0, tl = 0;
+  for (const Geom& g : gs) { tv += g.vec_blocks; tm += g.mv_blocks; tl += g.ls_blocks[1]; }
+  part = std::max((size_t)tv * (PCB_MAX_RESTART + 1), (size_t)std::max(tm, tl)) + 1;
   if (cudaMalloc(&G.dG, sizeof(Geom) * n) || cudaMalloc(&G.dS, sizeof(Slots) * n) ||
       cudaMalloc(&G.dSc, sizeof(Scal) * n) || cudaMalloc(&G.dAct, sizeof(int) * n) ||
       cudaMalloc(&G.dOff, sizeof(int) * batch_ints(n)) || cudaMalloc(&G.dPart, part * sizeof(double)) ||
@@ -1707,11 +1718,15 @@ int round_step(BGroup& G, const SolveCfg& c) {
     auto iter = [&](const Batch& Bx) -> int {
       CK(launch_matvec(Bx, PCB_OP_A, SL_Y, SL_Q, SL_R1, EPI_MINRES | (G.prec == PCB_MIXED ? EPI_FAST : 0)));
       CK(launch_reduce(Bx, Bx.off_mv, SS_MINRES_ALFA, c.tol, 0, 0));
-      CK(launch_axpby(Bx, AX_MINRES_R, SL_Q, SL_R2, SL_R1));
-      int r;
-      if ((r = apply_precond(p0, Bx, G.kind, G.prec, SL_R1, SL_YO))) return r;
-      CK(launch_dot(Bx, SL_R1, SL_YO));
-      CK(launch_reduce(Bx, Bx.off_vec, SS_MINRES_GIVENS, c.tol, 0, 0));
+      bool fused = false;
+      if (G.kind != PCB_PREC_NONE) CK(launch_precond_minres(Bx, G.kind, G.prec, SL_Q, SL_R2, SL_R1, SL_YO, &fused));
+      if (!fused) {
+        CK(launch_axpby(Bx, AX_MINRES_R, SL_Q, SL_R2, SL_R1));
+        int r;
+        if ((r = apply_precond(p0, Bx, G.kind, G.prec, SL_R1, SL_YO))) return r;
+        CK(launch_dot(Bx, SL_R1, SL_YO));
+      }
+      CK(launch_reduce(Bx, fused ? Bx.off_ls[1] : Bx.off_vec, SS_MINRES_GIVENS, c.tol, 0, 0));
       CK(launch_minres_wx(Bx, SL_Y, SL_W, SL_W2, SL_XI));
       CK(launch_swap(Bx, SL_R1, SL_R2, SL_Y, SL_YO, SL_W, SL_W2));
       return PCB_OK;
@@ -2167,10 +2182,14 @@ int srv_group_step(pcb_server* S, SrvGroup& G) {
     if (G.method == PCB_MINRES) {
       CK(launch_matvec(G.B, PCB_OP_A, SL_Y, SL_Q, SL_R1, EPI_MINRES | (prec == PCB_MIXED ? EPI_FAST : 0)));
       CK(launch_reduce(G.B, G.B.off_mv, SS_MINRES_ALFA, tol, 0, 0));
-      CK(launch_axpby(G.B, AX_MINRES_R, SL_Q, SL_R2, SL_R1));
-      if ((rc = precond(SL_R1, SL_YO))) return rc;
-      CK(launch_dot(G.B, SL_R1, SL_YO));
-      CK(launch_reduce(G.B, G.B.off_vec, SS_MINRES_GIVENS, tol, 0, 0));
+      bool fused = false;
+      CK(launch_precond_minres(G.B, G.kind, prec, SL_Q, SL_R2, SL_R1, SL_YO, &fused));
+      if (!fused) {
+        CK(launch_axpby(G.B, AX_MINRES_R, SL_Q, SL_R2, SL_R1));
+        if ((rc = precond(SL_R1, SL_YO))) return rc;
+        CK(launch_dot(G.B, SL_R1, SL_YO));
+      }
+      CK(launch_reduce(G.B, fused ? G.B.off_ls[1] : G.B.off_vec, SS_MINRES_GIVENS, tol, 0, 0));
       CK(launch_minres_wx(G.B, SL_Y, SL_W, SL_W2, SL_XI));
       if ((rc = srv_read(G, st))) return rc;
       for (int k = 0; k < G.cap; ++k) {

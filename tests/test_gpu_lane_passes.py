@@ -104,3 +104,19 @@ def test_batch_of_different_zetas(P):
         assert np.linalg.norm(b - op.matvec_A(prob, x.cpu().numpy())) <= 1.5e-8 * np.linalg.norm(b)
         _, alone = P.batch_solve([gp], [dev(b)], tol=1e-8)
         assert alone[0]["iterations"] == info["iterations"]
+
+
+@pytest.mark.parametrize("N,n", [(15, 2), (31, 16), (47, 8), (95, 4), (127, 4), (191, 2), (255, 4), (383, 2), (511, 2)])
+def test_residual_update_and_inner_product_in_the_passes(P, N, n):
+    """A mixed solve forms MINRES's residual in pass 1 and its inner product in pass 5; a profiled one
+    keeps both in kernels of their own.  The same residual bit for bit, the sum in another order: iterates
+    after 5 steps agree to the rounding of beta carried through the recurrences (1e-12), for sizes with
+    every line length and ragged tiles."""
+    prob = ds.Problem(N, n, 1.0, 1e-2)
+    b = dev(ds.rhs_minres(prob, synth.random_target(N, n, seed=9), synth.manufactured_source(N, n))
+            + 1e-3 * synth.random_vector(2 * prob.m * n, seed=10))
+    gp = P.Problem(N, n, 1.0, 1e-2, precision="mixed")
+    fused, i1 = gp.solve(b, fixed_iterations=5)
+    apart, i2 = gp.solve(b, fixed_iterations=5, profile=True)
+    assert i1["launches"] < i2["launches"]
+    assert_close(fused.cpu().numpy(), apart.cpu().numpy(), 1e-12)
