@@ -123,6 +123,54 @@ __global__ void __launch_bounds__(256) k_minres_wx(const Geom* __restrict__ G, c
   }
 }
 
+// The updates of two iterations k, k+1 at once (coefficients wp*: iteration k, w*: k+1):
+//   u_k     = y_k     + wpc2 u_{k-2} + wpc1 u_{k-1}   -> slot w2
+//   u_{k+1} = y_{k+1} + wc2 u_{k-1} + wc1 u_k         -> slot w;   x += wpcx u_k + wcx u_{k+1}
+// 64 B a value for both instead of 96: the update of a single iteration is bound by HBM, and its FP64
+// operations (three a value and iteration) fit under the two-iteration traffic (N = 511, n = 512: two launches
+// of 2.02 ms -> one of 3.12).
+__global__ void __launch_bounds__(256) k_minres_wx2(const Geom* __restrict__ G, const Slots* __restrict__ S,
+                                                    const Scal* __restrict__ Sc, const int* __restrict__ off, int count,
+                                                    const int* __restrict__ active, int sy0, int sy1, int sw, int sw2,
+                                                    int sx) {
+  INST_PROLOGUE
+  const Scal& c = Sc[inst];
+  const double* __restrict__ y0 = S[inst].v[sy0];
+  const double* __restrict__ y1 = S[inst].v[sy1];
+  double* __restrict__ w = S[inst].v[sw];
+  double* __restrict__ w2 = S[inst].v[sw2];
+  double* __restrict__ x = S[inst].v[sx];
+  const double p1 = c.wpc1, p2 = c.wpc2, px = c.wpcx, c1 = c.wc1, c2 = c.wc2, cx = c.wcx;
+  long long e = e0;
+  for (; e + 3 * stride < len; e += 4 * stride) {       // four values in flight
+    double s[4], t[4], a[4], b[4], z[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      s[q] = y0[e + q * stride];
+      t[q] = y1[e + q * stride];
+      a[q] = w2[e + q * stride];
+      b[q] = w[e + q * stride];
+      z[q] = x[e + q * stride];
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      s[q] = fma(p1, b[q], fma(p2, a[q], s[q]));
+      t[q] = fma(c1, s[q], fma(c2, b[q], t[q]));
+      w2[e + q * stride] = s[q];
+      w[e + q * stride] = t[q];
+      x[e + q * stride] = fma(cx, t[q], fma(px, s[q], z[q]));
+    }
+  }
+  for (; e < len; e += stride) {
+    const double b = w[e];
+    const double u = fma(p1, b, fma(p2, w2[e], y0[e]));
+    const double t = fma(c1, u, fma(c2, b, y1[e]));
+    w2[e] = u;
+    w[e] = t;
+    x[e] = fma(cx, t, fma(px, u, x[e]));
+  }
+}
+
 // Classical Gram-Schmidt over JB basis vectors, two values per thread and step (vectors have even
 // length and basis vectors start on 16 bytes).  Both kernels are bound by FP64 issue (one FMA per value
 // and vector: 63 us a vector at N = 255, n = 256, against 39 us of HBM) as long as enough loads are in
@@ -283,6 +331,7 @@ __device__ void scalar_step(Scal& c, int step, double v, double tol, int j, int 
       c.phi = c.cs * c.phibar;
       c.phibar = c.sn * c.phibar;
       // coefficients of k_minres_wx: w_{k-1} = ws1 u_{k-1}, w_{k-2} = ws2 u_{k-2}
+      c.wpc1 = c.wc1; c.wpc2 = c.wc2; c.wpcx = c.wcx;
       c.wc1 = -c.oldb * c.delta * c.ws1;
       c.wc2 = -c.oldb * c.oldeps * c.ws2;
       c.ws2 = c.ws1;
@@ -461,6 +510,10 @@ cudaError_t launch_axpby(const Batch& B, int mode, int sx, int sy, int sz) {
 }
 cudaError_t launch_minres_wx(const Batch& B, int sy, int sw, int sw2, int sx) {
   k_minres_wx<<<B.tot_vec, 256, 0, B.stream>>>(B.G, B.S, B.Sc, B.off_vec, B.count, B.active, sy, sw, sw2, sx);
+  return cudaGetLastError();
+}
+cudaError_t launch_minres_wx2(const Batch& B, int sy0, int sy1, int sw, int sw2, int sx) {
+  k_minres_wx2<<<B.tot_vec, 256, 0, B.stream>>>(B.G, B.S, B.Sc, B.off_vec, B.count, B.active, sy0, sy1, sw, sw2, sx);
   return cudaGetLastError();
 }
 // Arnoldi index j >= 0: the kernel of exactly j + 1 vectors.  j < 0 (per-instance indices, at most jmax when

@@ -179,6 +179,7 @@ struct Scal {
   double beta1, bnorm, est;
   double rf;                        // -alfa/beta: residual update r1 = q + rf r2
   double wc1, wc2, wcx, ws1, ws2;   // direction update in unscaled form (k_minres_wx)
+  double wpc1, wpc2, wpcx;          // the iteration before's (k_minres_wx2)
   // reductions land here
   double dot0, dot1;
   // GMRES

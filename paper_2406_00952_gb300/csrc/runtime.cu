@@ -56,6 +56,7 @@ cudaError_t launch_dot(const Batch& B, int sa, int sb);
 cudaError_t launch_reduce(const Batch& B, const int* off, int step, double tol, int j, int restart);
 cudaError_t launch_axpby(const Batch& B, int mode, int sx, int sy, int sz);
 cudaError_t launch_minres_wx(const Batch& B, int sy, int sw, int sw2, int sx);
+cudaError_t launch_minres_wx2(const Batch& B, int sy0, int sy1, int sw, int sw2, int sx);
 // j < 0: each instance at its own Arnoldi index (from Scal), all of them <= jmax when jmax >= 0
 cudaError_t launch_multidot(const Batch& B, int svbase, int j, int sw, int jmax = -1);
 cudaError_t launch_reduce_multi(const Batch& B, int j, int pass, int jmax = -1);
@@ -134,11 +135,11 @@ struct pcb_problem {
   Slots* hSpin = nullptr;         // pinned staging for slot uploads
   Batch B;
   double* host_io = nullptr;      // device staging for pcb_solve_host (b, x)
-  // CUDA graph of one MINRES iteration (captured on a private stream, replayed on `stream`)
+  // CUDA graphs of a MINRES iteration (captured on a private stream, replayed on `stream`)
   cudaStream_t cap_stream = nullptr;
-  cudaGraphExec_t git = nullptr;
+  cudaGraphExec_t git[2] = {};    // first and second iteration of a pair (minres_iter_launches)
   int git_kind = -1, git_prec = -1, git_sx = -1;
-  long long git_launches = 0;
+  long long git_launches[2] = {};
   // CUDA graphs of the FGMRES Arnoldi steps, one per index j, for one (preconditioner, precision,
   // restart) setting
   cudaGraphExec_t garn[PCB_MAX_RESTART] = {};
@@ -430,7 +431,7 @@ void pcb_destroy(pcb_problem* p) {
   cudaFreeHost(p->hSc);
   cudaFreeHost(p->hSpin);
   cudaFree(p->host_io);
-  if (p->git) cudaGraphExecDestroy(p->git);
+  for (cudaGraphExec_t e : p->git) if (e) cudaGraphExecDestroy(e);
   for (cudaGraphExec_t e : p->garn) if (e) cudaGraphExecDestroy(e);
   if (p->cap_stream) cudaStreamDestroy(p->cap_stream);
   cudaFree(p->dtol);
@@ -792,30 +793,34 @@ static int read_scal(const Batch& B, Scal* host, int count) {
 // Single-instance MINRES on slot rhs -> slot x (both set by the caller).  Returns iterations via sc.
 #define LC(p) (++(p)->launches, 0) ? cudaSuccess :
 
-// One MINRES iteration's launches: product with the Lanczos epilogue, scalar steps, residual
-// update, preconditioner, inner product, direction/solution update, slot rotation.  Every kernel
-// takes its scalars and vector pointers from device memory (Scal, Slots, the tolerance in
-// B.tols), so one launch sequence serves every iteration and can be replayed from a graph.
-static int minres_iter_launches(pcb_problem* p, const Batch& B, const SolveCfg& c, int s_x) {
+// One MINRES iteration's launches: product with the Lanczos epilogue, scalar steps, residual update,
+// preconditioner, inner product, slot rotation.  The direction/solution updates are made for two iterations
+// at a time (k_minres_wx2): the first of a pair leaves its y_k in slot YO, which the second therefore may not
+// overwrite; it puts y_{k+2} over q, which is dead once the residual has been formed.
+//   first:  y -> Y = y_{k+1}, YO = y_k;       second: Y = y_{k+2}, Q = the buffer of y_{k+1}.
+// Every kernel takes its scalars and vector pointers from device memory (Scal, Slots, the tolerance in
+// B.tols), so one launch sequence serves every pair and can be replayed from a graph.
+static int minres_iter_launches(pcb_problem* p, const Batch& B, const SolveCfg& c, int s_x, bool second) {
   int rc;
+  const int s_out = second ? SL_Q : SL_YO;
   CK(P_matvec(p, B, PCB_OP_A, SL_Y, SL_Q, SL_R1, EPI_MINRES | (c.prec == PCB_MIXED ? EPI_FAST : 0)));
   CK(LC(p) launch_reduce(B, B.off_mv, SS_MINRES_ALFA, c.tol, 0, 0));
   // residual update, preconditioner and inner product: in the preconditioner's own passes where it can be
   // (a profiled solve times the preconditioner, so it keeps them apart)
   bool fused = false;
   if (!p->prof && c.kind != PCB_PREC_NONE && !p->g.mg_route)
-    CK(launch_precond_minres(B, c.kind, c.prec, SL_Q, SL_R2, SL_R1, SL_YO, &fused));
+    CK(launch_precond_minres(B, c.kind, c.prec, SL_Q, SL_R2, SL_R1, s_out, &fused));
   if (fused) {
     p->launches += precond_launch_count(false, c.kind);
     p->prec_applies += 1;
   } else {
     CK(LC(p) launch_axpby(B, AX_MINRES_R, SL_Q, SL_R2, SL_R1));
-    if ((rc = P_precond(p, B, c.kind, c.prec, SL_R1, SL_YO))) return rc;
-    CK(LC(p) launch_dot(B, SL_R1, SL_YO));
+    if ((rc = P_precond(p, B, c.kind, c.prec, SL_R1, s_out))) return rc;
+    CK(LC(p) launch_dot(B, SL_R1, s_out));
   }
   CK(LC(p) launch_reduce(B, fused ? B.off_ls[1] : B.off_vec, SS_MINRES_GIVENS, c.tol, 0, 0));
-  CK(LC(p) launch_minres_wx(B, SL_Y, SL_W, SL_W2, s_x));
-  CK(LC(p) launch_swap(B, SL_R1, SL_R2, SL_Y, SL_YO, SL_W, SL_W2));
+  if (second) CK(LC(p) launch_minres_wx2(B, SL_YO, SL_Y, SL_W, SL_W2, s_x));
+  CK(LC(p) launch_swap(B, SL_R1, SL_R2, SL_Y, s_out, -1, -1));
   return PCB_OK;
 }
 
@@ -854,11 +859,12 @@ static cudaGraphExec_t capture_launches(pcb_problem* p, const Batch& B, F&& issu
   return exec;
 }
 
-static bool capture_minres_iter(pcb_problem* p, const Batch& B, const SolveCfg& c, int s_x) {
-  if (p->git) { cudaGraphExecDestroy(p->git); p->git = nullptr; }
-  p->git = capture_launches(p, B, [&](const Batch& Bc) { return minres_iter_launches(p, Bc, c, s_x); },
-                            &p->git_launches);
-  if (!p->git) return false;
+static bool capture_minres_iter(pcb_problem* p, const Batch& B, const SolveCfg& c, int s_x, bool second) {
+  if (p->git_kind != c.kind || p->git_prec != c.prec || p->git_sx != s_x)
+    for (cudaGraphExec_t& e : p->git) if (e) { cudaGraphExecDestroy(e); e = nullptr; }
+  p->git[second] = capture_launches(p, B, [&](const Batch& Bc) { return minres_iter_launches(p, Bc, c, s_x, second); },
+                                    &p->git_launches[second]);
+  if (!p->git[second]) return false;
   p->git_kind = c.kind; p->git_prec = c.prec; p->git_sx = s_x;
   return true;
 }
@@ -886,6 +892,16 @@ static int minres_single(pcb_problem* p, const SolveCfg& c, int s_b, int s_x, Sc
   if (hs->bnorm == 0.0 || !hs->active) { *conv_out = true; *relres_out = 0.0; return PCB_OK; }
   const int limit = c.fixed > 0 ? c.fixed : c.maxit;
   bool checking = false;
+  bool second = false;              // the next iteration is the second of a pair: the first's update is pending
+  // the update of an iteration whose pair does not follow (y in slot YO since the rotation)
+  auto flush = [&]() -> int {
+    if (!second) return PCB_OK;
+    CK(LC(p) launch_minres_wx(B, SL_YO, SL_W, SL_W2, s_x));
+    CK(LC(p) launch_swap(B, SL_W, SL_W2, -1, -1, -1, -1));
+    std::swap(p->hS.v[SL_W], p->hS.v[SL_W2]);
+    second = false;
+    return PCB_OK;
+  };
   // the iterations read the tolerance from the device, so a captured graph serves every sweep
   if (!p->dtol && cudaMalloc(&p->dtol, sizeof(double)) != cudaSuccess) { cudaGetLastError(); p->dtol = nullptr; }
   Batch Bt = B;
@@ -896,26 +912,28 @@ static int minres_single(pcb_problem* p, const SolveCfg& c, int s_b, int s_x, Sc
   }
   for (int it = 0; it < limit; ++it) {
     // the first iteration runs directly (one-time kernel attribute setup happens there)
-    if (graph && it >= 1 && !(p->git && p->git_kind == c.kind && p->git_prec == c.prec && p->git_sx == s_x))
-      graph = capture_minres_iter(p, Bt, c, s_x);
+    if (graph && it >= 1 &&
+        !(p->git[second] && p->git_kind == c.kind && p->git_prec == c.prec && p->git_sx == s_x))
+      graph = capture_minres_iter(p, Bt, c, s_x, second);
     if (graph && it >= 1) {
-      CK(cudaGraphLaunch(p->git, p->stream));
-      p->launches += p->git_launches;
+      CK(cudaGraphLaunch(p->git[second], p->stream));
+      p->launches += p->git_launches[second];
       p->prec_applies += 1;
       p->matvecs += 1;
       p->matvecs_inner += c.prec == PCB_MIXED ? 1 : 0;
-    } else if ((rc = minres_iter_launches(p, Bt, c, s_x))) {
+    } else if ((rc = minres_iter_launches(p, Bt, c, s_x, second))) {
       return rc;
     }
     std::swap(p->hS.v[SL_R1], p->hS.v[SL_R2]);
-    std::swap(p->hS.v[SL_Y], p->hS.v[SL_YO]);
-    std::swap(p->hS.v[SL_W], p->hS.v[SL_W2]);
+    std::swap(p->hS.v[SL_Y], p->hS.v[second ? SL_Q : SL_YO]);
+    second = !second;
     if ((rc = read_scal(B, hs, 1))) return rc;
     *it_out = it + 1;
     if (hs->flags & 4) return PCB_ERR_NONFINITE;
     if (hs->flags & 2) return PCB_ERR_BREAKDOWN;
     if (c.fixed > 0) continue;
     if ((hs->flags & 1) || checking) {
+      if ((rc = flush())) return rc;
       // an inner solve of a refinement sweep ends at its first estimate below the tolerance; the
       // sweep then measures the true residual of the outer system itself
       if (!c.check_true) { *relres_out = hs->est; return PCB_OK; }
@@ -928,6 +946,7 @@ static int minres_single(pcb_problem* p, const SolveCfg& c, int s_b, int s_x, Sc
       checking = true;
     }
   }
+  if ((rc = flush())) return rc;
   if (!c.check_true) { *relres_out = hs->est; return PCB_OK; }
   CK(P_matvec(p, B, PCB_OP_A, s_x, SL_Q, s_b, EPI_RESID));
   CK(LC(p) launch_reduce(B, B.off_mv, SS_NORM, c.tol, 0, 0));
@@ -1426,7 +1445,7 @@ int pcb_autotune(pcb_problem* p, int kind, int reps, pcb_tune_info* info) {
   }
   if ((rc = install(cands[best_k]))) return done(rc);
   // captured iterations launch the kernels of the old configuration
-  if (p->git) { cudaGraphExecDestroy(p->git); p->git = nullptr; }
+  for (cudaGraphExec_t& e : p->git) if (e) { cudaGraphExecDestroy(e); e = nullptr; }
   for (cudaGraphExec_t& e : p->garn) if (e) { cudaGraphExecDestroy(e); e = nullptr; }
   p->git_kind = p->garn_kind = -1;
   {
@@ -1464,7 +1483,7 @@ int pcb_tune_select(pcb_problem* p, int candidate, pcb_tune_info* info) {
     int rc = fill_batch(p->B, std::vector<Geom>(1, p->g), p->doff, p->stream, staging);
     if (rc) return rc;
     CK(cudaStreamSynchronize(p->stream));
-    if (p->git) { cudaGraphExecDestroy(p->git); p->git = nullptr; }
+    for (cudaGraphExec_t& e : p->git) if (e) { cudaGraphExecDestroy(e); e = nullptr; }
     for (cudaGraphExec_t& e : p->garn) if (e) { cudaGraphExecDestroy(e); e = nullptr; }
     p->git_kind = p->garn_kind = -1;
   }
