@@ -101,7 +101,6 @@ __device__ __forceinline__ Epi make_epi(int kind, const Scal* sc) {
 // took as long as the first.
 constexpr int kMvThreads = 128;
 __host__ __device__ int tw_patches(int N);
-static_assert(32 * 4 == kMvThreads, "two-word product: one thread per point of a 32 x 4 patch");
 
 void matvec_shape(Geom& g) {
   const int ncb = (g.m + kMvThreads - 1) / kMvThreads;
@@ -383,7 +382,11 @@ __global__ void __launch_bounds__(kMvThreads, 7) k_matvec_march(const Geom* __re
 // ------------------------------------------------------------------------------------------
 namespace tw {
 
-constexpr int kI = 32, kJ = 4;                  // patch: x1 by x2 points (kI * kJ = kMvThreads)
+constexpr int kI = 32, kJ = 4;                  // patch: x1 by x2 points, one thread each
+constexpr int kThreads = kI * kJ;
+// Eight blocks an SM (64 registers).  With 7 and 6 blocks the N = 511, n = 256 step takes 971 and 1004 us instead
+// of 967; patches of 32 x 8 points split a fifth fewer halo points but wait longer at the barrier: 1028 us.
+constexpr int kBlocks = 8;
 constexpr int kW = kI + 2, kH = kJ + 2;         // with the halo
 constexpr int kSlots = kW * kH;
 constexpr int kHalo = 2 * kI + 2 * kJ;          // halo points (corners unused)
@@ -430,21 +433,28 @@ __device__ __forceinline__ void acc(f2& h, f2& l, f2 ph, f2 pl) {
   l = add(l, add(e, pl));
 }
 
-// x 2^-k split into two FP32 words (b20 = (896 + k) << 20, the FP64 exponent bias of the scaled
-// value): hi = the leading 24 bits of the significand, lo = the next 23 (both truncated), so
-// |x 2^-k - hi - lo| < 2^-46 |x 2^-k|.  The second word is the difference of two FP32 numbers of
-// the same binade (exact).  Scaled values below 2^-103 and FP64 subnormals become 0.
-__device__ __forceinline__ void split(double x, int b20, float& hi, float& lo) {
+// x 2^-k split into two FP32 words: hi = the leading 24 bits of the significand, lo = the next 23 (both
+// truncated), so |x 2^-k - hi - lo| < 2^-46 |x 2^-k|.  The second word is the difference of two FP32
+// numbers of the same binade (exact).  Scaled values below 2^-103 and FP64 subnormals become 0, values
+// beyond the FP32 range NaN.
+struct Scale {
+  unsigned bias;           // 896 + k at the FP32 exponent's place (modulo 2^32)
+  unsigned low, range;     // |x| (high word) of the smallest covered value, and the covered span
+};
+__device__ __forceinline__ Scale scale_of(int k) {
+  // FP32 exponents 24 .. 254 of the scaled value, and FP64 exponents 1 .. 2046
+  const int lo = max(920 + k, 1), hi = min(1151 + k, 2047);
+  return Scale{(unsigned)(896 + k) << 23, (unsigned)lo << 20, (unsigned)max(hi - lo, 0) << 20};
+}
+__device__ __forceinline__ void split(double x, const Scale& s, float& hi, float& lo) {
   const unsigned hw = (unsigned)__double2hiint(x), lw = (unsigned)__double2loint(x);
-  const unsigned sgn = hw & 0x80000000u;
-  const int u = (int)(hw & 0x7fffffffu) - b20;             // FP32 exponent field at bit 20
-  const unsigned hb = (__funnelshift_l(lw, (unsigned)u, 3) & 0x7fffffffu) | sgn;
-  const unsigned s3 = ((unsigned)u << 3) - (23u << 23);     // unit of the second word
-  const unsigned one = (s3 & 0x7f800000u) | sgn;
+  const unsigned t = hw & 0x7fffffffu;
+  const unsigned m = __funnelshift_l(lw, hw, 3) - s.bias;
+  const unsigned hb = (m & 0x7fffffffu) | (hw & 0x80000000u);
+  const unsigned one = (hb & 0xff800000u) - (23u << 23);    // sign and unit of the second word
   const float l = __fsub_rn(__uint_as_float(one | ((lw >> 6) & 0x007fffffu)), __uint_as_float(one));
-  // a normal FP64 value whose scaled exponent lies in [-103, 127] (zeros and FP64 subnormals give 0)
-  const bool ok = (hw & 0x7ff00000u) != 0u && (unsigned)(u - (24 << 20)) < (231u << 20);
-  hi = ok ? __uint_as_float(hb) : (u >= (255 << 20) ? __uint_as_float(0x7fc00000u) : 0.f);
+  const bool ok = t - s.low < s.range;
+  hi = ok ? __uint_as_float(hb) : (t < s.low ? 0.f : __uint_as_float(0x7fc00000u));
   lo = ok ? l : 0.f;
 }
 // exact FP64 value of an FP32 word (subnormal words give 0; infinities and NaN are kept)
@@ -526,7 +536,7 @@ __device__ __forceinline__ double matvec_tw_block(const Geom& g, int lb, int op,
   const bool use_aux = e.c != 0.0;
   const int ka = use_aux ? binade(sc.oldb) : 0;
   const double sgd = e.s * pow2(ky), kpd = e.c * pow2(ka);
-  const int by = (896 + ky) * (1 << 20), ba = (896 + ka) * (1 << 20);
+  const Scale by = scale_of(ky), ba = scale_of(ka);
   float w0, w1;
   split_rn(sgd, w0, w1);
   const f2 SGh = pk(w0, w0), SGl = pk(w1, w1), nSG = pk(-w0, -w0);
@@ -642,7 +652,7 @@ __device__ __forceinline__ double matvec_tw_block(const Geom& g, int lb, int op,
   return ((widen(dh.x) + widen(dh.y)) + (widen(dl.x) + widen(dl.y))) * sgd;
 }
 
-__global__ void __launch_bounds__(kMvThreads) k_matvec_tw(const Geom* __restrict__ G, const Slots* __restrict__ S,
+__global__ void __launch_bounds__(tw::kThreads, tw::kBlocks) k_matvec_tw(const Geom* __restrict__ G, const Slots* __restrict__ S,
                                                    Scal* __restrict__ Sc, const int* __restrict__ off, int count,
                                                    const int* __restrict__ active, int op, int x_slot, int out_slot,
                                                    int aux_slot, double* __restrict__ partial) {
@@ -692,7 +702,7 @@ cudaError_t launch_matvec(const Batch& B, int op, int x_slot, int out_slot, int 
   const int kind = epi & (EPI_FAST - 1), fast = (epi & EPI_FAST) && kind == EPI_MINRES;
   const int set = fast ? B.mv_set_fast : B.mv_set;
   if (set & MV_TW)
-    k_matvec_tw<<<B.tot_mv, kMvThreads, 0, B.stream>>>(B.G, B.S, B.Sc, B.off_mv, B.count, B.active, op, x_slot,
+    k_matvec_tw<<<B.tot_mv, tw::kThreads, 0, B.stream>>>(B.G, B.S, B.Sc, B.off_mv, B.count, B.active, op, x_slot,
                                                        out_slot, aux_slot, B.partial);
   if (set & MV_MARCH)
     k_matvec_march<<<B.tot_mv, kMvThreads, 0, B.stream>>>(B.G, B.S, B.Sc, B.off_mv, B.count, B.active, op, x_slot,
