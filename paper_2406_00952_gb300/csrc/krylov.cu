@@ -427,7 +427,7 @@ __global__ void __launch_bounds__(32) k_backsub(int count, const int* __restrict
 __global__ void __launch_bounds__(512) k_reduce(const int* __restrict__ off, int count, const int* __restrict__ active,
                                                 const double* __restrict__ partial, Scal* Sc,
                                                 int step, double tol, const double* __restrict__ tols, int j,
-                                                int restart) {
+                                                int restart, Slots* S, int a0, int s0, int a1, int s1) {
   const int inst = blockIdx.x;
   if (inst >= count) return;
   if (active && !active[inst]) return;
@@ -450,6 +450,11 @@ __global__ void __launch_bounds__(512) k_reduce(const int* __restrict__ off, int
     arnoldi_step(Sc[inst], total, tl, j < 0 ? Sc[inst].j : j);
   } else if (threadIdx.x == 0) {
     scalar_step(Sc[inst], step, s, tl, j, restart);
+    if (a0 >= 0) {
+      double** v = S[inst].v;
+      double* t = v[a0]; v[a0] = v[s0]; v[s0] = t;
+      t = v[a1]; v[a1] = v[s1]; v[s1] = t;
+    }
   }
 }
 
@@ -499,9 +504,11 @@ cudaError_t launch_dot(const Batch& B, int sa, int sb) {
   k_dot<<<B.tot_vec, 256, 0, B.stream>>>(B.G, B.S, B.off_vec, B.count, B.active, sa, sb, B.partial);
   return cudaGetLastError();
 }
-cudaError_t launch_reduce(const Batch& B, const int* off, int step, double tol, int j, int restart) {
+cudaError_t launch_reduce(const Batch& B, const int* off, int step, double tol, int j, int restart, int a0, int b0,
+                          int a1, int b1) {
   // one block size for every instance: the order of its sum must not depend on the batch it is in
-  k_reduce<<<B.count, 512, 0, B.stream>>>(off, B.count, B.active, B.partial, B.Sc, step, tol, B.tols, j, restart);
+  k_reduce<<<B.count, 512, 0, B.stream>>>(off, B.count, B.active, B.partial, B.Sc, step, tol, B.tols, j, restart,
+                                          B.S, a0, b0, a1, b1);
   return cudaGetLastError();
 }
 cudaError_t launch_axpby(const Batch& B, int mode, int sx, int sy, int sz) {

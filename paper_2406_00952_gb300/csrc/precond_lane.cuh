@@ -505,43 +505,45 @@ __global__ void __launch_bounds__(spatial_threads<R, M>(), spatial_blocks<R, M>(
 //   part of the twiddle after it: exp(-i pi t / n) W_n^{t k1} = exp(-i pi t (2 k1 + 1) / n), a table
 //   of 2n entries.
 //   General zeta (GZ): the halves are two lines; a thread holds both at the same k1.
-// B = 1 (n <= 16): the whole line sits in one thread.
+// B = 1 (short lines): the whole line sits in one thread.
 // ------------------------------------------------------------------------------------------
-template <int n> struct TimeShape;
-template <> struct TimeShape<2> { static constexpr int A = 2, B = 1; };
-template <> struct TimeShape<4> { static constexpr int A = 4, B = 1; };
-template <> struct TimeShape<8> { static constexpr int A = 8, B = 1; };
-template <> struct TimeShape<16> { static constexpr int A = 16, B = 1; };
-template <> struct TimeShape<32> { static constexpr int A = 8, B = 4; };
-template <> struct TimeShape<64> { static constexpr int A = 8, B = 8; };
-template <> struct TimeShape<128> { static constexpr int A = 16, B = 8; };
-template <> struct TimeShape<256> { static constexpr int A = 16, B = 16; };
-template <> struct TimeShape<512> { static constexpr int A = 32, B = 16; };
-template <> struct TimeShape<1024> { static constexpr int A = 32, B = 32; };
+template <typename R, int n> struct TimeShape { static constexpr int A = n, B = 1; };       // n <= 4
+// FP32 lines of 8 and 16 steps stay in one thread; FP64 ones are spread, because a small problem is bound
+// by the serial FP64 work of a warp (about 76 cycles an instruction): N = 15, n = 16 26 -> 12 us
+template <> struct TimeShape<float, 8> { static constexpr int A = 8, B = 1; };
+template <> struct TimeShape<float, 16> { static constexpr int A = 16, B = 1; };
+template <> struct TimeShape<double, 8> { static constexpr int A = 4, B = 2; };
+template <> struct TimeShape<double, 16> { static constexpr int A = 8, B = 2; };
+template <typename R> struct TimeShape<R, 32> { static constexpr int A = 8, B = 4; };
+template <typename R> struct TimeShape<R, 64> { static constexpr int A = 8, B = 8; };
+template <typename R> struct TimeShape<R, 128> { static constexpr int A = 16, B = 8; };
+template <typename R> struct TimeShape<R, 256> { static constexpr int A = 16, B = 16; };
+template <typename R> struct TimeShape<R, 512> { static constexpr int A = 32, B = 16; };
+template <typename R> struct TimeShape<R, 1024> { static constexpr int A = 32, B = 32; };
 
 // columns per tile: an exchange near 64 KB (two lines a column for general zeta)
 template <typename R, int n, bool GZ>
 constexpr int time_lanes() {
   constexpr int vals = n * (GZ ? 2 : 1) * (int)(sizeof(R) / 4);
-  return n <= 16 ? 32 : vals <= 128 ? 32 : vals <= 512 ? 16 : vals <= 1024 ? (sizeof(R) == 8 ? 16 : 8) : 8;
+  return TimeShape<R, n>::B == 1 ? 32 : vals <= 128 ? 32 : vals <= 512 ? 16 : vals <= 1024 ? (sizeof(R) == 8 ? 16 : 8) : 8;
 }
 // lane groups: one per pair of rows (zeta = pi: A/2 pairs) or per row (general zeta: A), at most one per
-// first step (B); the one-thread lines run four tiles a block
+// first step (B) on long lines; the one-thread lines run four tiles a block
 template <typename R, int n, bool GZ>
 constexpr int time_groups() {
-  constexpr int A = TimeShape<n>::A, B = TimeShape<n>::B;
+  constexpr int A = TimeShape<R, n>::A, B = TimeShape<R, n>::B;
   constexpr int rows = GZ ? A : A / 2;
-  return B == 1 ? 1 : rows < B ? rows : B;
+  return B == 1 ? 1 : n <= 16 || rows < B ? rows : B;
 }
 template <typename R, int n, bool GZ>
 constexpr int time_threads() { return time_groups<R, n, GZ>() * time_lanes<R, n, GZ>(); }
 template <typename R, int n, bool GZ>
 constexpr size_t time_smem() {
-  return TimeShape<n>::B == 1 ? 0 : (size_t)(GZ ? 2 : 1) * n * time_lanes<R, n, GZ>() * sizeof(cx<R>);
+  return TimeShape<R, n>::B == 1 ? 0 : (size_t)(GZ ? 2 : 1) * n * time_lanes<R, n, GZ>() * sizeof(cx<R>);
 }
 template <typename R, int n, bool GZ>
 constexpr int time_blocks_per_sm() {
-  constexpr int th = TimeShape<n>::B == 1 ? 128 : time_threads<R, n, GZ>();
+  constexpr int th = TimeShape<R, n>::B == 1 ? 128 : time_threads<R, n, GZ>();
   if (sizeof(R) == 8) return th <= 128 ? 2 : 1;
   return n >= 1024 ? 1 : n <= 64 && th <= 128 ? 8 : th <= 128 || n == 128 ? 4 : th <= 256 ? 2 : 1;
 }
@@ -599,11 +601,11 @@ __device__ __forceinline__ void solve_halves(int kind, cx<R>& V1, cx<R>& V2, cx<
 }
 
 template <typename R, int n, bool GZ>
-__global__ void __launch_bounds__((TimeShape<n>::B == 1 ? 128 : time_threads<R, n, GZ>()), (time_blocks_per_sm<R, n, GZ>()))
+__global__ void __launch_bounds__((TimeShape<R, n>::B == 1 ? 128 : time_threads<R, n, GZ>()), (time_blocks_per_sm<R, n, GZ>()))
     k_lane_time(const Geom* __restrict__ G, const Slots* __restrict__ S, const int* __restrict__ off, int count, Sel sel,
                 int kind, int in_sel, int out_sel, int) {
   using T = cx<R>;
-  constexpr int A = TimeShape<n>::A, B = TimeShape<n>::B, NG = time_groups<R, n, GZ>(), LT = time_lanes<R, n, GZ>();
+  constexpr int A = TimeShape<R, n>::A, B = TimeShape<R, n>::B, NG = time_groups<R, n, GZ>(), LT = time_lanes<R, n, GZ>();
   constexpr int H = GZ ? 2 : 1;
   extern __shared__ __align__(16) unsigned char lane_smem[];
   const int inst = find_inst(off, count, blockIdx.x);
@@ -831,7 +833,7 @@ template <typename R, int n, bool GZ>
 cudaError_t time_pass_n(const Batch& B, Sel sel, int kind, int in_sel, int out_sel) {
   constexpr int p = sizeof(R) == 4;
   static DeviceInt resident;
-  return launch(k_lane_time<R, n, GZ>, resident, B.tot_lt[p], TimeShape<n>::B == 1 ? 128 : time_threads<R, n, GZ>(),
+  return launch(k_lane_time<R, n, GZ>, resident, B.tot_lt[p], TimeShape<R, n>::B == 1 ? 128 : time_threads<R, n, GZ>(),
                 time_smem<R, n, GZ>(), B.stream, B.G, (const Slots*)B.S, B.off_lt[p], B.count, sel, kind, in_sel, out_sel);
 }
 

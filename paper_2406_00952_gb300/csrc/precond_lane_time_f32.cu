@@ -29,7 +29,7 @@ int lines(int M) {
 // tile shapes for the launch counts: lines per spatial tile, columns per time tile, time tiles per block
 int lane_space_lines(int M, int p) { return p ? lines<float>(M) : lines<double>(M); }
 int lane_time_columns(int n, bool gz, int p) { return p ? columns<float>(n, gz) : columns<double>(n, gz); }
-int lane_time_tiles(int n) { return n <= 16 ? 4 : 1; }
+int lane_time_tiles(int n, int p) { return n <= (p ? 16 : 4) ? 4 : 1; }
 
 cudaError_t lane_time_f32(const Batch& B, Sel sel, int n, bool gz, int kind, int in_sel, int out_sel) {
   switch (n) {

@@ -53,7 +53,9 @@ static cudaError_t copy_host(double* dst, const double* src, size_t n, bool to_d
                          st);
 }
 cudaError_t launch_dot(const Batch& B, int sa, int sb);
-cudaError_t launch_reduce(const Batch& B, const int* off, int step, double tol, int j, int restart);
+// a0 >= 0: after the step, exchange the instance's slots a0, b0 and a1, b1
+cudaError_t launch_reduce(const Batch& B, const int* off, int step, double tol, int j, int restart, int a0 = -1,
+                          int b0 = -1, int a1 = -1, int b1 = -1);
 cudaError_t launch_axpby(const Batch& B, int mode, int sx, int sy, int sz);
 cudaError_t launch_minres_wx(const Batch& B, int sy, int sw, int sw2, int sx);
 cudaError_t launch_minres_wx2(const Batch& B, int sy0, int sy1, int sw, int sw2, int sx);
@@ -83,7 +85,7 @@ int pipe_time_cols(int n, int zeta_pi);
 int pipe_dst_lines(int L);
 int lane_space_lines(int M, int p);
 int lane_time_columns(int n, bool gz, int p);
-int lane_time_tiles(int n);
+int lane_time_tiles(int n, int p);
 cudaError_t upload_constants();
 struct TableLayout { size_t kap, mud, muf, twdd, twdf, twtd, twtf, pred, pref, ax, ay, dg, ms, bytes; };
 cudaError_t mg_setup(Geom& g, void* ws, const double* a_edges_host, double a0);
@@ -181,8 +183,10 @@ bool make_plan(int M, FftPlan& p) {
   return r == 1;
 }
 
+// blocks of 256 threads of the vector kernels: a value a thread on short vectors, up to a block an SM, then
+// eight values a thread (N = 15, n = 16: 4 blocks -> 29; the kernels 7-8 -> 4-5 us each)
 int vec_blocks_for(long long len) {
-  long long b = (len + 2047) / 2048;
+  long long b = std::max(std::min<long long>((len + 255) / 256, 152), (len + 2047) / 2048);
   if (b > 2432) b = 2432;
   if (b < 1) b = 1;
   return (int)b;
@@ -204,7 +208,7 @@ void set_lane_shapes(Geom& g) {
     g.lane_tm[p] = tm;
     const int lines = lane_space_lines(g.M, p), cols = lane_time_columns(g.n, !g.zeta_pi, p);
     g.ls_blocks[p] = g.n * ((g.N + lines - 1) / lines);
-    const int tiles = g.N * ((g.N + cols - 1) / cols), per = lane_time_tiles(g.n);
+    const int tiles = g.N * ((g.N + cols - 1) / cols), per = lane_time_tiles(g.n, p);
     g.lt_blocks[p] = (tiles + per - 1) / per;
     g.dst_blocks_i[p] = g.dst_blocks_j[p] = g.time_blocks[p] = 0;
     if (p == 1) {        // the padded layout (two FP32 buffers) of the FP32 passes
@@ -818,9 +822,9 @@ static int minres_iter_launches(pcb_problem* p, const Batch& B, const SolveCfg& 
     if ((rc = P_precond(p, B, c.kind, c.prec, SL_R1, s_out))) return rc;
     CK(LC(p) launch_dot(B, SL_R1, s_out));
   }
-  CK(LC(p) launch_reduce(B, fused ? B.off_ls[1] : B.off_vec, SS_MINRES_GIVENS, c.tol, 0, 0));
-  if (second) CK(LC(p) launch_minres_wx2(B, SL_YO, SL_Y, SL_W, SL_W2, s_x));
-  CK(LC(p) launch_swap(B, SL_R1, SL_R2, SL_Y, s_out, -1, -1));
+  // (the scalar step also rotates the slots; y_{k+1} of the update then sits in slot Q)
+  CK(LC(p) launch_reduce(B, fused ? B.off_ls[1] : B.off_vec, SS_MINRES_GIVENS, c.tol, 0, 0, SL_R1, SL_R2, SL_Y, s_out));
+  if (second) CK(LC(p) launch_minres_wx2(B, SL_YO, SL_Q, SL_W, SL_W2, s_x));
   return PCB_OK;
 }
 
