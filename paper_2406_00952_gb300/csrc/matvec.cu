@@ -124,18 +124,19 @@ void matvec_shape(Geom& g) {
   }
 }
 
-// theta < 1, one role of one block of columns: T x1 - alpha x2 marching forward in time (role 0) or
-// alpha x1 + T^T x2 marching backward (role 1).  With u the marched half, the recurrence
+// theta < 1 (HALF: theta = 1/2), one role of one block of columns: T x1 - alpha x2 marching forward in
+// time (role 0) or alpha x1 + T^T x2 marching backward (role 1).  With u the marched half, the recurrence
 // z_t = (u_t - (1-theta) z_{t-1})/theta gives (B_n u)_t = z_t - z_{t-1} = (u_t - z_{t-1})/theta, so
 //     out = (1/theta + diagonal) u_t - z_{t-1}/theta - (off-diagonal sum) -/+ alpha (other half)
 // and, for theta = 1/2, z_t = 2 u_t - z_{t-1}: eight FP64 operations per value for a constant
-// coefficient (ten when the difference z_t - z_{t-1} and the stencil are formed on their own).  The
-// kernel is bound by FP64 issue: N = 255, n = 256 0.84 -> 0.70 ms, 72% of the measured FP64 rate.
+// coefficient (ten when the difference z_t - z_{t-1} and the stencil are formed on their own).  HALF is a
+// template argument because a choice at run time computes both forms of z.  The kernel is bound by
+// FP64 issue: N = 255, n = 256 0.84 -> 0.57 ms, 90% of the measured FP64 rate.
 // A small grid has too few columns to fill the device with one thread each.  Its time range is split
 // in g.mv_chunks parts: a first sweep marches every part from z = 0, the carries combine through
 // (-(1-theta)/theta)^length, and the second sweep computes the values (GMRES
 // solve at N = 63, n = 64: 2.71 -> 2.28 ms, its products having taken 84 us each).
-template <bool VAR>
+template <bool VAR, bool HALF>
 __device__ __forceinline__ double march_block(const Geom& g, int lb, int op, const double* __restrict__ x,
                                               double* __restrict__ out, const double* __restrict__ aux, const Epi& e) {
   __shared__ double carry[kMvThreads];
@@ -149,14 +150,13 @@ __device__ __forceinline__ double march_block(const Geom& g, int lb, int op, con
   const int t0 = role ? n - 1 - s0 : s0;
   const long long step = role ? -(long long)m : m;
   const double th = g.theta, ith = 1.0 / th, r = (1.0 - th) * ith;
-  const bool half = r == 1.0;                              // theta = 1/2
   const long long at0 = (long long)t0 * m + (ok ? col : 0);
   const double* __restrict__ u = x + (role ? mn : 0) + at0;
   double z = 0.0;
   if (chunks > 1) {
     const double* v = u;
     if (ok)
-      for (int k = 0; k < len; ++k, v += step) z = half ? fma(ith, *v, -z) : fma(-r, z, ith * *v);
+      for (int k = 0; k < len; ++k, v += step) z = HALF ? fma(ith, *v, -z) : fma(-r, z, ith * *v);
     carry[threadIdx.x] = z;
     __syncthreads();
     double pw = 1.0;
@@ -199,7 +199,7 @@ __device__ __forceinline__ double march_block(const Geom& g, int lb, int op, con
     }
     o = fma(-ith, z, o);
     o = fma(alpha, *w, o);
-    z = half ? fma(ith, uc, -z) : fma(-r, z, ith * uc);
+    z = HALF ? fma(ith, uc, -z) : fma(-r, z, ith * uc);
     out[a] = epi_apply(e, o, aux, x, a, part);
   }
   return part;
@@ -348,7 +348,11 @@ __global__ void __launch_bounds__(kMvThreads, 7) k_matvec_march(const Geom* __re
   const int lb = blockIdx.x - off[inst];
   const double* __restrict__ x = S[inst].v[x_slot];
   double* __restrict__ out = S[inst].v[out_slot];
-  double part = g.var_a ? march_block<true>(g, lb, op, x, out, aux, e) : march_block<false>(g, lb, op, x, out, aux, e);
+  double part;
+  if (g.theta == 0.5)
+    part = g.var_a ? march_block<true, true>(g, lb, op, x, out, aux, e) : march_block<false, true>(g, lb, op, x, out, aux, e);
+  else
+    part = g.var_a ? march_block<true, false>(g, lb, op, x, out, aux, e) : march_block<false, false>(g, lb, op, x, out, aux, e);
   if (epi_kind == EPI_MINRES) part *= e.s;
   if (partial && epi_kind != EPI_PLAIN) block_reduce_store(part, partial + blockIdx.x);
 }
