@@ -25,7 +25,7 @@
 #include <cstring>
 #include <vector>
 
-#include "fft_reg.cuh"
+#include "precond_lane.cuh"
 
 namespace pcb {
 
@@ -689,145 +689,232 @@ __global__ void k_mg_axpy(long long len, const cx<R>* __restrict__ src, cx<R>* _
 // ------------------------------------------------------------------------------------------
 // time passes around the multigrid
 // ------------------------------------------------------------------------------------------
-template <typename R> __device__ __forceinline__ const cx<R>* twt_(const Geom& g);
-template <> __device__ __forceinline__ const float2* twt_<float>(const Geom& g) { return g.twt_f; }
-template <> __device__ __forceinline__ const double2* twt_<double>(const Geom& g) { return g.twt_d; }
-template <typename R> __device__ __forceinline__ const cx<R>* pre_(const Geom& g);
-template <> __device__ __forceinline__ const float2* pre_<float>(const Geom& g) { return g.pre_f; }
-template <> __device__ __forceinline__ const double2* pre_<double>(const Geom& g) { return g.pre_d; }
+// The transforms of precond_lane.cuh (n = A B, two register steps with one exchange) with one column per
+// lane: the forward pass ends in the decoupled right-hand sides, the inverse one begins with the
+// recoupling.  A slot pair (r, n-1-r) is held by one thread, so the coupling needs no second exchange, and
+// every global access of a half warp is a full 128-byte line.  Both are bound by HBM and by the
+// conversions between FP64 and FP32, half of which go to the integer pipe (f32_convert.cuh).  The kernels
+// before them gave a column to a warp and wrote the slots of one column side by side, m values apart:
+// N = 255, n = 256, FP32 197 + 172 us, now 88 + 90 us (the traffic alone takes 59 us each).
+template <typename R, int n>
+constexpr int mg_time_columns() { return lane::TimeShape<R, n>::B == 1 ? 128 : lane::time_lanes<R, n, false>(); }
+template <typename R, int n>
+constexpr int mg_time_threads() { return lane::TimeShape<R, n>::B == 1 ? 128 : lane::time_threads<R, n, false>(); }
 
-__host__ __device__ __forceinline__ int padded_len_mg(int len) { return (len + (len >> 5) + 1) | 1; }
-
-// Shared-memory radix-2 Stockham-free DFT of one column of length n by a single warp-group:
-// the time passes here handle one column per warp with the register/shuffle FFT.
-template <typename R, int Q>
-__device__ __forceinline__ void col_fft(cx<R>* line, int t, int P, const cx<R>* __restrict__ tw, bool inv) {
-  using T = cx<R>;
-  LaneStages<T, R> st;
-  lane_stages<T, R>(st, t, P, inv);
-  T x[Q];
+// x[q] = the pair of halves at p[q step] in R, q < A
+template <typename R, int A>
+__device__ __forceinline__ void load_pairs(cx<R>* x, const double* __restrict__ p, const double* __restrict__ p2,
+                                           long long step) {
+  if constexpr (sizeof(R) == 8) {
 #pragma unroll
-  for (int q = 0; q < Q; ++q) x[q] = line[pidx(t + P * q)];
-  __syncwarp();
-  reg_dft<T, R, Q>(x, inv);
+    for (int q = 0; q < A; ++q) x[q] = mk<R>(p[q * step], p2[q * step]);
+  } else {
+    unsigned rare = 0;
 #pragma unroll
-  for (int k1 = 1; k1 < Q; ++k1) {
-    T w = __ldg(&tw[t * k1]);
-    if (inv) w.y = -w.y;
-    x[pos<Q>(k1)] = cmul(x[pos<Q>(k1)], w);
+    for (int q = 0; q < A; ++q) x[q] = mk<R>((R)p[q * step], (R)d2f_plain(p2[q * step], rare));
+    if (rare) {
+#pragma unroll
+      for (int q = 0; q < A; ++q) x[q].y = (R)p2[q * step];
+    }
   }
-  lane_dif<T, R, Q>(x, P, st);
-  __syncwarp();
-  const int k2 = bitrev(t, P);
-#pragma unroll
-  for (int k1 = 0; k1 < Q; ++k1) line[pidx(k1 + Q * k2)] = x[pos<Q>(k1)];
-  __syncwarp();
+}
+template <typename R>
+__device__ __forceinline__ void store_pair(double* p, double* p2, cx<R> v, unsigned& rare) {
+  *p = (double)v.x;
+  if constexpr (sizeof(R) == 8) *p2 = v.y;
+  else *p2 = f2d_plain(v.y, rare);
+}
+
+// right-hand sides of slot r (systems 2r and 2r + 1) from C_r and C_{n-1-r}
+template <typename R>
+__device__ __forceinline__ void put_slot(cx<R>* __restrict__ rhs, const cx<R>* __restrict__ tab, int kind, long long m,
+                                         int r, cx<R> Cr, cx<R> Cq) {
+  using T = cx<R>;
+  Cq = cconj(Cq);
+  const T F1 = cscale(cadd(Cr, Cq), (R)0.5);
+  const T F2 = cmul_mi(cscale(csub(Cr, Cq), (R)0.5));
+  T T1 = F1, T2 = F2;
+  if (kind == 2) {   // W^{-1} [F1; F2], W = [[1, M], [M, 1]]
+    const T M = __ldg(&tab[4 * r + 1]);
+    const R inv = __ldg(&tab[4 * r + 2]).x;
+    T1 = cscale(csub(F1, cmul(M, F2)), inv);
+    T2 = cscale(csub(F2, cmul(M, F1)), inv);
+    T2 = cconj(T2);   // second component: solved as the conjugate system with D1
+  }
+  rhs[2 * r * m] = T1;
+  rhs[(2 * r + 1) * m] = T2;
+}
+// C_r and C_{n-1-r} from the solutions of slot r
+template <typename R>
+__device__ __forceinline__ void get_slot(const cx<R>* __restrict__ z, const cx<R>* __restrict__ tab, int kind,
+                                         long long m, int r, cx<R>& Cr, cx<R>& Cq) {
+  using T = cx<R>;
+  const T Z1 = z[2 * r * m];
+  T Z2 = z[(2 * r + 1) * m];
+  T U1 = Z1, U2 = Z2;
+  if (kind == 2) {
+    Z2 = cconj(Z2);
+    const T M = __ldg(&tab[4 * r + 1]);
+    U1 = cadd(Z1, cmul(M, Z2));
+    U2 = cadd(cmul(M, Z1), Z2);
+  }
+  Cr = cadd(U1, cmul_pi(U2));
+  Cq = cadd(cconj(U1), cmul_pi(cconj(U2)));
 }
 
 // forward: v (FP64, 2 halves) -> right-hand sides of the n systems (slot r < n/2: 2r and 2r+1)
-template <typename R, int Q>
-__global__ void __launch_bounds__(256) k_mg_time_fwd(const Geom* __restrict__ G, const Slots* __restrict__ S,
-                                                     int in_slot, const cx<R>* __restrict__ tab, int kind,
-                                                     cx<R>* __restrict__ rhs, int cpw) {
+template <typename R, int n>
+__global__ void __launch_bounds__((mg_time_threads<R, n>()), (lane::time_blocks_per_sm<R, n, false>()))
+    k_mg_time_fwd(const Geom* __restrict__ G, const Slots* __restrict__ S, int in_slot, const cx<R>* __restrict__ tab,
+                  int kind, cx<R>* __restrict__ rhs) {
   using T = cx<R>;
-  const Geom& g = G[0];
-  const int n = g.n, m = g.m, ls = padded_len_mg(n);
-  const long long mn = g.mn;
-  const double* __restrict__ x = S[0].v[in_slot];
+  constexpr int A = lane::TimeShape<R, n>::A, B = lane::TimeShape<R, n>::B;
+  constexpr int LT = mg_time_columns<R, n>(), NG = mg_time_threads<R, n>() / LT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* tile = (T*)smem_raw;
-  const int P = n / Q, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lpw = 32 / P;
-  const int t = lane % P;
-  const int cols_per_block = (blockDim.x >> 5) * lpw * cpw;
-  const int c0 = blockIdx.x * cols_per_block;
-  for (int e = threadIdx.x; e < cols_per_block * n; e += blockDim.x) {
-    const int tt = e / cols_per_block, l = e - tt * cols_per_block;
-    const int col = c0 + l;
-    T v = mk<R>(0, 0);
-    if (col < m) {
-      const long long a = (long long)tt * m + col;
-      v = cmul(mk<R>((R)x[a], (R)x[mn + a]), __ldg(&pre_<R>(g)[tt]));
+  const Geom& g = G[0];
+  const int m = g.m, l = threadIdx.x % LT, grp = threadIdx.x / LT;
+  const int col = blockIdx.x * LT + l;
+  const bool ok = col < m;
+  const double* __restrict__ x0 = S[0].v[in_slot] + (ok ? col : m - 1);
+  const T* __restrict__ pre = lane::twist<R>(g);
+  rhs += col;
+  if constexpr (B == 1) {
+    T x[A];
+    load_pairs<R, A>(x, x0, x0 + g.mn, m);
+#pragma unroll
+    for (int t = 0; t < n; ++t) x[t] = cmul(x[t], __ldg(&pre[t]));
+    reg_dft<T, R, A>(x, false);
+    if (ok) {
+#pragma unroll
+      for (int r = 0; r < n / 2; ++r) put_slot<R>(rhs, tab, kind, m, r, x[pos<A>(r)], x[pos<A>(n - 1 - r)]);
     }
-    tile[l * ls + pidx(tt)] = v;
-  }
-  __syncthreads();
-  const int half = n / 2;
-  for (int k = 0; k < cpw; ++k) {
-    const int l = (warp * cpw + k) * lpw + lane / P;
-    T* line = tile + l * ls;
-    col_fft<R, Q>(line, t, P, twt_<R>(g), false);
-    const int col = c0 + l;
-    if (col < m) {
-      for (int r = t; r < half; r += P) {
-        const T Cr = line[pidx(r)], Cq = cconj(line[pidx(n - 1 - r)]);
-        const T F1 = cscale(cadd(Cr, Cq), (R)0.5);
-        const T F2 = cmul_mi(cscale(csub(Cr, Cq), (R)0.5));
-        T T1 = F1, T2 = F2;
-        if (kind == 2) {   // W^{-1} [F1; F2], W = [[1, M], [M, 1]]
-          const T M = tab[4 * r + 1];
-          const R inv = tab[4 * r + 2].x;
-          T1 = cscale(csub(F1, cmul(M, F2)), inv);
-          T2 = cscale(csub(F2, cmul(M, F1)), inv);
-          T2 = cconj(T2);   // second component: solved as the conjugate system with D1
+  } else {
+    T* ex = (T*)smem_raw + l;                        // position e of the line: ex[e LT]
+#pragma unroll 1
+    for (int t = grp; t < B; t += NG) {
+      const double* __restrict__ p = x0 + (long long)t * m;
+      T x[A];
+      load_pairs<R, A>(x, p, p + g.mn, (long long)B * m);
+#pragma unroll
+      for (int q = 1; q < A; ++q) x[q] = cmul(x[q], root64<R>(q * (32 / A)));
+      reg_dft<T, R, A>(x, false);
+#pragma unroll
+      for (int k = 0; k < A; ++k) ex[(t * A + k) * LT] = x[pos<A>(k)];
+    }
+    __syncthreads();
+    // rows k1 and A-1-k1, whose twiddles are conjugate up to a shift by one slot (see k_lane_time)
+#pragma unroll 1
+    for (int k1 = grp; k1 < A / 2; k1 += NG) {
+      T va[B], vb[B];
+#pragma unroll
+      for (int t = 0; t < B; ++t) {
+        va[t] = ex[(t * A + k1) * LT];
+        vb[t] = ex[(t * A + A - 1 - k1) * LT];
+        if (t) {
+          const T w = __ldg(&pre[t * (2 * k1 + 1)]);
+          va[t] = cmul(va[t], w);
+          vb[t] = lane::mulc(vb[t], w);
         }
-        rhs[(long long)(2 * r) * m + col] = T1;
-        rhs[(long long)(2 * r + 1) * m + col] = T2;
+      }
+      reg_dft<T, R, B>(va, false);
+      reg_dft<T, R, B>(vb, false);
+      if (ok) {
+#pragma unroll
+        for (int k2 = 0; k2 < B; ++k2) {             // slot k1 + A k2 or its partner, whichever is below n/2
+          const T Xa = va[pos<B>(k2)], Xb = vb[pos<B>((B - k2) % B)];
+          if (k2 < B / 2) put_slot<R>(rhs, tab, kind, m, k1 + A * k2, Xa, Xb);
+          else put_slot<R>(rhs, tab, kind, m, n - 1 - k1 - A * k2, Xb, Xa);
+        }
       }
     }
   }
 }
 
 // inverse: solutions of the n systems -> P^{-1} v (FP64, 2 halves)
-template <typename R, int Q>
-__global__ void __launch_bounds__(256) k_mg_time_inv(const Geom* __restrict__ G, const Slots* __restrict__ S,
-                                                     int out_slot, const cx<R>* __restrict__ tab, int kind,
-                                                     const cx<R>* __restrict__ z, int cpw) {
+template <typename R, int n>
+__global__ void __launch_bounds__((mg_time_threads<R, n>()), (lane::time_blocks_per_sm<R, n, false>()))
+    k_mg_time_inv(const Geom* __restrict__ G, const Slots* __restrict__ S, int out_slot, const cx<R>* __restrict__ tab,
+                  int kind, const cx<R>* __restrict__ z) {
   using T = cx<R>;
-  const Geom& g = G[0];
-  const int n = g.n, m = g.m, ls = padded_len_mg(n);
-  const long long mn = g.mn;
-  double* __restrict__ y = S[0].v[out_slot];
+  constexpr int A = lane::TimeShape<R, n>::A, B = lane::TimeShape<R, n>::B;
+  constexpr int LT = mg_time_columns<R, n>(), NG = mg_time_threads<R, n>() / LT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* tile = (T*)smem_raw;
-  const int P = n / Q, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lpw = 32 / P;
-  const int t = lane % P;
-  const int cols_per_block = (blockDim.x >> 5) * lpw * cpw;
-  const int c0 = blockIdx.x * cols_per_block;
-  const int half = n / 2;
-  for (int e = threadIdx.x; e < cols_per_block * half; e += blockDim.x) {
-    const int r = e / cols_per_block, l = e - r * cols_per_block;
-    const int col = c0 + l;
-    T U1 = mk<R>(0, 0), U2 = mk<R>(0, 0);
-    if (col < m) {
-      const T Z1 = z[(long long)(2 * r) * m + col];
-      T Z2 = z[(long long)(2 * r + 1) * m + col];
-      if (kind == 2) {
-        Z2 = cconj(Z2);
-        const T M = tab[4 * r + 1];
-        U1 = cadd(Z1, cmul(M, Z2));
-        U2 = cadd(cmul(M, Z1), Z2);
-      } else {
-        U1 = Z1; U2 = Z2;
+  const Geom& g = G[0];
+  const int m = g.m, l = threadIdx.x % LT, grp = threadIdx.x / LT;
+  const int col = blockIdx.x * LT + l;
+  const bool ok = col < m;
+  double* __restrict__ y = S[0].v[out_slot] + col;
+  double* __restrict__ y2 = y + g.mn;
+  const T* __restrict__ pre = lane::twist<R>(g);
+  z += ok ? col : m - 1;
+  const R sc = (R)1 / (R)n;
+  unsigned rare = 0;
+  if constexpr (B == 1) {
+    T x[A];
+#pragma unroll
+    for (int r = 0; r < n / 2; ++r) get_slot<R>(z, tab, kind, m, r, x[r], x[n - 1 - r]);
+    reg_dft<T, R, A>(x, true);
+    if (!ok) return;
+#pragma unroll
+    for (int t = 0; t < n; ++t) {
+      x[pos<A>(t)] = cscale(lane::mulc(x[pos<A>(t)], __ldg(&pre[t])), sc);
+      store_pair<R>(y + (long long)t * m, y2 + (long long)t * m, x[pos<A>(t)], rare);
+    }
+    if (rare) {
+#pragma unroll
+      for (int t = 0; t < n; ++t) y2[(long long)t * m] = (double)x[pos<A>(t)].y;
+    }
+  } else {
+    T* ex = (T*)smem_raw + l;
+#pragma unroll 1
+    for (int k1 = grp; k1 < A / 2; k1 += NG) {
+      T za[B], zb[B];
+#pragma unroll
+      for (int k2 = 0; k2 < B; ++k2) {
+        T Xr, Xq;
+        if (k2 < B / 2) {
+          get_slot<R>(z, tab, kind, m, k1 + A * k2, Xr, Xq);
+          za[k2] = Xr;
+          zb[(B - k2) % B] = Xq;
+        } else {
+          get_slot<R>(z, tab, kind, m, n - 1 - k1 - A * k2, Xr, Xq);
+          za[k2] = Xq;
+          zb[(B - k2) % B] = Xr;
+        }
+      }
+      reg_dft<T, R, B>(za, true);
+      reg_dft<T, R, B>(zb, true);
+#pragma unroll
+      for (int t = 0; t < B; ++t) {
+        T a = za[pos<B>(t)], b = zb[pos<B>(t)];
+        if (t) {
+          const T w = __ldg(&pre[t * (2 * k1 + 1)]);
+          a = lane::mulc(a, w);
+          b = cmul(b, w);
+        }
+        ex[(t * A + k1) * LT] = cscale(a, sc);
+        ex[(t * A + A - 1 - k1) * LT] = cscale(b, sc);
       }
     }
-    tile[l * ls + pidx(r)] = cadd(U1, cmul_pi(U2));
-    tile[l * ls + pidx(n - 1 - r)] = cadd(cconj(U1), cmul_pi(cconj(U2)));
-  }
-  __syncthreads();
-  for (int k = 0; k < cpw; ++k) {
-    const int l = (warp * cpw + k) * lpw + lane / P;
-    col_fft<R, Q>(tile + l * ls, t, P, twt_<R>(g), true);
-  }
-  __syncthreads();
-  const R sc = (R)1 / (R)n;
-  for (int e = threadIdx.x; e < cols_per_block * n; e += blockDim.x) {
-    const int tt = e / cols_per_block, l = e - tt * cols_per_block;
-    const int col = c0 + l;
-    if (col < m) {
-      const T v = cscale(cmul(tile[l * ls + pidx(tt)], cconj(__ldg(&pre_<R>(g)[tt]))), sc);
-      const long long a = (long long)tt * m + col;
-      y[a] = (double)v.x;
-      y[mn + a] = (double)v.y;
+    __syncthreads();
+    if (!ok) return;
+#pragma unroll 1
+    for (int t = grp; t < B; t += NG) {
+      T x[A];
+#pragma unroll
+      for (int k = 0; k < A; ++k) x[k] = ex[(t * A + k) * LT];
+      reg_dft<T, R, A>(x, true);
+      rare = 0;
+#pragma unroll
+      for (int q = 0; q < A; ++q) {
+        const long long at = (long long)(t + B * q) * m;
+        if (q) x[pos<A>(q)] = lane::mulc(x[pos<A>(q)], root64<R>(q * (32 / A)));
+        store_pair<R>(y + at, y2 + at, x[pos<A>(q)], rare);
+      }
+      if (rare) {
+#pragma unroll
+        for (int q = 0; q < A; ++q) y2[(long long)(t + B * q) * m] = (double)x[pos<A>(q)].y;
+      }
     }
   }
 }
@@ -903,7 +990,7 @@ static void vcycle(const MgHost& h, const cx<R>* tab, int kind, int l, const cx<
   }
 }
 
-template <typename R, int Q>
+template <typename R, int n>
 static cudaError_t mg_apply(const Batch& B, const Geom& g, const MgHost& h, int kind, int cycles, int in_slot,
                             int out_slot) {
   using T = cx<R>;
@@ -914,16 +1001,15 @@ static cudaError_t mg_apply(const Batch& B, const Geom& g, const MgHost& h, int 
   T* r0 = (T*)F.a[0];
   T* z0 = (T*)h.zfine;
   T* x0 = (T*)h.xfine;
-  const int P = g.n / Q, lpw = 32 / P, cpw = 2;   // two lines per warp: 16-column tiles, 128-byte runs of FP64
-  const int cols = 8 * lpw * cpw;
-  const size_t smem = (size_t)cols * padded_len_mg(g.n) * sizeof(T);
+  constexpr int cols = mg_time_columns<R, n>(), threads = mg_time_threads<R, n>();
+  constexpr size_t smem = lane::time_smem<R, n, false>();
   static DeviceOnce once;
   once([] {
-    cudaFuncSetAttribute(k_mg_time_fwd<R, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    return cudaFuncSetAttribute(k_mg_time_inv<R, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    cudaFuncSetAttribute(k_mg_time_fwd<R, n>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return cudaFuncSetAttribute(k_mg_time_inv<R, n>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   });
   const unsigned tb = (unsigned)((g.m + cols - 1) / cols);
-  k_mg_time_fwd<R, Q><<<tb, 256, smem, st>>>(B.G, B.S, in_slot, tab, kind, r0, cpw);
+  k_mg_time_fwd<R, n><<<tb, threads, smem, st>>>(B.G, B.S, in_slot, tab, kind, r0);
   g_mg_launches += 2;
   for (int c = 0; c < cycles; ++c) {
     if (c == 0) {
@@ -935,19 +1021,23 @@ static cudaError_t mg_apply(const Batch& B, const Geom& g, const MgHost& h, int 
       g_mg_launches += 2;
     }
   }
-  k_mg_time_inv<R, Q><<<tb, 256, smem, st>>>(B.G, B.S, out_slot, tab, kind, z0, cpw);
+  k_mg_time_inv<R, n><<<tb, threads, smem, st>>>(B.G, B.S, out_slot, tab, kind, z0);
   return cudaGetLastError();
 }
 
 template <typename R>
 static cudaError_t mg_dispatch(const Batch& B, const Geom& g, const MgHost& h, int kind, int cycles, int in_slot,
                                int out_slot) {
-  switch (g.time_q) {
-    case 1: return mg_apply<R, 1>(B, g, h, kind, cycles, in_slot, out_slot);
+  switch (g.n) {
     case 2: return mg_apply<R, 2>(B, g, h, kind, cycles, in_slot, out_slot);
     case 4: return mg_apply<R, 4>(B, g, h, kind, cycles, in_slot, out_slot);
     case 8: return mg_apply<R, 8>(B, g, h, kind, cycles, in_slot, out_slot);
     case 16: return mg_apply<R, 16>(B, g, h, kind, cycles, in_slot, out_slot);
+    case 32: return mg_apply<R, 32>(B, g, h, kind, cycles, in_slot, out_slot);
+    case 64: return mg_apply<R, 64>(B, g, h, kind, cycles, in_slot, out_slot);
+    case 128: return mg_apply<R, 128>(B, g, h, kind, cycles, in_slot, out_slot);
+    case 256: return mg_apply<R, 256>(B, g, h, kind, cycles, in_slot, out_slot);
+    case 512: return mg_apply<R, 512>(B, g, h, kind, cycles, in_slot, out_slot);
     default: return cudaErrorInvalidValue;
   }
 }
