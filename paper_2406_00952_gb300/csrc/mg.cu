@@ -438,84 +438,178 @@ __global__ void __launch_bounds__(256) k_mg_resid(MgLevel L, const cx<R>* __rest
   res[o1 + pt] = r1;
 }
 
-// tau K z at grid point (gi, gj) of a Dirichlet level from a shared-memory window whose row
-// pitch is WX and in which (gi, gj) sits at (li, lj): the arithmetic of tauKz
-template <typename R>
-__device__ __forceinline__ cx<R> tauKz_win(const MgLevel& L, const cx<R>* zs, int WX, int li, int lj, int gi,
-                                           int gj) {
-  const int N = L.N;
-  const R* ax = Coef<R>::ax(L) + (long long)gj * (N + 1);
-  const R* ay = Coef<R>::ay(L);
-  const cx<R> c = zs[lj * WX + li];
-  cx<R> s = mk<R>(0, 0);
-  if (gi > 0) s = cadd(s, cscale(zs[lj * WX + li - 1], ax[gi]));
-  if (gi < N - 1) s = cadd(s, cscale(zs[lj * WX + li + 1], ax[gi + 1]));
-  if (gj > 0) s = cadd(s, cscale(zs[(lj - 1) * WX + li], ay[(long long)gj * N + gi]));
-  if (gj < N - 1) s = cadd(s, cscale(zs[(lj + 1) * WX + li], ay[(long long)(gj + 1) * N + gi]));
-  const R d = Coef<R>::dg(L)[gj * N + gi];
-  return csub(cscale(c, d), s);
+// The fused smoothing of a Dirichlet level.  A block takes a 32 x 16 tile of both systems of a slot, with
+// the two systems' values side by side (one 16-byte access for both).  Every point's stencil coefficients
+// and Jacobi weight are formed once for both systems and the weight once for both sweeps: with 32 x 8
+// tiles, a weight per sweep and separate systems, instructions bound the pre-smoothing (level 0 at N = 255,
+// n = 256: 181 us, now 136; its traffic alone takes 59 us).
+template <typename R> struct alignas(4 * sizeof(R)) Duo { cx<R> v[2]; };
+namespace tile {
+constexpr int TX = 32, TY = 16, WX2 = TX + 4, WY2 = TY + 4, WX1 = TX + 2, WY1 = TY + 2;
+}
+static dim3 tile_grid(int N, int nslot) {
+  return dim3((unsigned)((N + tile::TX - 1) / tile::TX), (unsigned)((N + tile::TY - 1) / tile::TY), (unsigned)nslot);
 }
 
-// The pre-smoothing of a Dirichlet level (two sweeps, the first from zero) and the residual of its
-// result in one launch.  A block takes a 32 x 8 tile of both systems of a slot: it loads the
-// right-hand sides on the tile with a halo of two points, runs the first sweep there, the second on
-// the tile with a halo of one, and forms the residual on the tile, all in shared memory; it writes
-// the smoothed solution and the residual.  The same per-point arithmetic as the three separate
-// launches (jacobi_pt, resid_pt), which read and wrote 8 full grids where this moves 3.
+// (mu I + tau K) z at grid point (gi, gj) from a window of row pitch WX whose entry (gi, gj) is zs[at], for both
+// systems: the arithmetic of tauKz.  The window holds zeros outside the grid.
+template <typename R, int WX>
+__device__ __forceinline__ Duo<R> shifted_win(const MgLevel& L, cx<R> mu, const Duo<R>* zs, int at, int gi, int gj) {
+  const int N = L.N, pt = gj * N + gi;
+  const R* ax = Coef<R>::ax(L) + pt + gj;              // rows of N + 1 edges
+  const R* ay = Coef<R>::ay(L) + pt;
+  const R al = __ldg(ax), ar = __ldg(ax + 1), ad = __ldg(ay), au = __ldg(ay + N), d = __ldg(Coef<R>::dg(L) + pt);
+  const Duo<R> c = zs[at], l = zs[at - 1], r = zs[at + 1], dn = zs[at - WX], up = zs[at + WX];
+  Duo<R> o;
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    cx<R> s = cscale(l.v[k], al);
+    s = cadd(s, cscale(r.v[k], ar));
+    s = cadd(s, cscale(dn.v[k], ad));
+    s = cadd(s, cscale(up.v[k], au));
+    o.v[k] = cadd(cmul(mu, c.v[k]), csub(cscale(c.v[k], d), s));
+  }
+  return o;
+}
+// one damped Jacobi update from the window
+template <typename R, int WX>
+__device__ __forceinline__ Duo<R> jacobi_win(const MgLevel& L, cx<R> mu, cx<R> dinv, const Duo<R>& r, const Duo<R>* zs,
+                                             int at, int gi, int gj, R w) {
+  const Duo<R> Az = shifted_win<R, WX>(L, mu, zs, at, gi, gj), c = zs[at];
+  Duo<R> o;
+#pragma unroll
+  for (int k = 0; k < 2; ++k) o.v[k] = cadd(c.v[k], cscale(cmul(csub(r.v[k], Az.v[k]), dinv), w));
+  return o;
+}
+
+// The pre-smoothing (two sweeps, the first from zero) and the residual of its result: the right-hand sides
+// on the tile with a halo of two points, the first sweep there, the second with a halo of one, and the
+// residual on the tile.  Reads one grid and writes two, where the separate launches moved eight.
 template <typename R>
 __global__ void __launch_bounds__(256) k_mg_presmooth(MgLevel L, const cx<R>* __restrict__ tab, int kind,
                                                       const cx<R>* __restrict__ rhs, cx<R>* __restrict__ zout,
                                                       cx<R>* __restrict__ res, R w) {
   using C = cx<R>;
-  constexpr int TX = 32, TY = 8, WX2 = TX + 4, WY2 = TY + 4, WX1 = TX + 2, WY1 = TY + 2;
-  __shared__ C r2[2][WX2 * WY2], z1[2][WX2 * WY2], z2[2][WX1 * WY1];
+  using namespace tile;
+  __shared__ Duo<R> r2[WX2 * WY2], z1[WX2 * WY2], z2[WX1 * WY1];
+  __shared__ C di[WX2 * WY2];
   const int N = L.N, nn = N * N;
   const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, tid = threadIdx.y * TX + threadIdx.x;
-  const int b = 2 * blockIdx.z;
-  const C mu = shift_of<R>(tab, b, kind);
-  const long long o0 = (long long)b * nn;
+  const C mu = shift_of<R>(tab, 2 * blockIdx.z, kind);
+  const long long o0 = 2LL * blockIdx.z * nn, o1 = o0 + nn;
   const C zero = mk<R>(0, 0);
-  // the right-hand sides and the first sweep (from zero) on the tile with a halo of 2
-  for (int e = tid; e < WX2 * WY2; e += TX * TY) {
+  for (int e = tid; e < WX2 * WY2; e += 256) {
     const int lj = e / WX2, li = e - lj * WX2, gi = x0 - 2 + li, gj = y0 - 2 + lj;
-    const bool in = gi >= 0 && gi < N && gj >= 0 && gj < N;
-    const C dinv = in ? jacobi_dinv<R>(L, mu, gj * N + gi) : zero;
+    Duo<R> r{{zero, zero}}, z{{zero, zero}};
+    C dinv = zero;
+    if (gi >= 0 && gi < N && gj >= 0 && gj < N) {
+      const int pt = gj * N + gi;
+      r.v[0] = rhs[o0 + pt];
+      r.v[1] = rhs[o1 + pt];
+      dinv = jacobi_dinv<R>(L, mu, pt);
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const C rv = in ? rhs[o0 + (long long)k * nn + gj * N + gi] : zero;
-      r2[k][e] = rv;
-      z1[k][e] = in ? cscale(cmul(rv, dinv), w) : zero;
+      for (int k = 0; k < 2; ++k) z.v[k] = cscale(cmul(r.v[k], dinv), w);
     }
+    r2[e] = r;
+    z1[e] = z;
+    di[e] = dinv;
   }
   __syncthreads();
-  // the second sweep on the tile with a halo of 1
-  for (int e = tid; e < WX1 * WY1; e += TX * TY) {
-    const int lj1 = e / WX1, li1 = e - lj1 * WX1, gi = x0 - 1 + li1, gj = y0 - 1 + lj1;
-    const int li = li1 + 1, lj = lj1 + 1;
-    const bool in = gi >= 0 && gi < N && gj >= 0 && gj < N;
-    const C dinv = in ? jacobi_dinv<R>(L, mu, gj * N + gi) : zero;
+  for (int e = tid; e < WX1 * WY1; e += 256) {
+    const int lj = e / WX1, li = e - lj * WX1, gi = x0 - 1 + li, gj = y0 - 1 + lj, at = (lj + 1) * WX2 + li + 1;
+    Duo<R> z{{zero, zero}};
+    if (gi >= 0 && gi < N && gj >= 0 && gj < N) z = jacobi_win<R, WX2>(L, mu, di[at], r2[at], z1, at, gi, gj, w);
+    z2[e] = z;
+  }
+  __syncthreads();
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      C v = zero;
-      if (in) {
-        const C zc = z1[k][lj * WX2 + li];
-        const C Az = cadd(cmul(mu, zc), tauKz_win<R>(L, z1[k], WX2, li, lj, gi, gj));
-        v = cadd(zc, cscale(cmul(csub(r2[k][lj * WX2 + li], Az), dinv), w));
+  for (int h = 0; h < 2; ++h) {
+    const int ty = threadIdx.y + 8 * h, gi = x0 + threadIdx.x, gj = y0 + ty;
+    if (gi < N && gj < N) {
+      const int at = (ty + 1) * WX1 + threadIdx.x + 1, pt = gj * N + gi;
+      const Duo<R> Az = shifted_win<R, WX1>(L, mu, z2, at, gi, gj), zc = z2[at];
+      const Duo<R> r = r2[(ty + 2) * WX2 + threadIdx.x + 2];
+      zout[o0 + pt] = zc.v[0];
+      zout[o1 + pt] = zc.v[1];
+      res[o0 + pt] = csub(r.v[0], Az.v[0]);
+      res[o1 + pt] = csub(r.v[1], Az.v[1]);
+    }
+  }
+}
+
+// The coarse correction and the two post-smoothing sweeps: z plus the prolonged correction on the tile with
+// a halo of two points, one sweep with a halo of one, the second on the tile.  Reads two grids and a
+// quarter and writes one, where the separate launches moved eight and a quarter (level 0 at N = 255,
+// n = 256: 48 + 2 x 93 us, now 180; its traffic alone takes 64).  `base` (a further cycle, whose z corrects
+// base): the result is added there and not written to zout.
+template <typename R>
+__global__ void __launch_bounds__(256) k_mg_postsmooth(MgLevel L, const cx<R>* __restrict__ tab, int kind,
+                                                       const cx<R>* __restrict__ rhs, const cx<R>* __restrict__ zin,
+                                                       const cx<R>* __restrict__ coarse, cx<R>* __restrict__ zout,
+                                                       cx<R>* __restrict__ base, R w) {
+  using C = cx<R>;
+  using namespace tile;
+  constexpr int CX = TX / 2 + 3, CY = TY / 2 + 3;      // coarse points -2 .. TX/2 of the tile's corner
+  __shared__ Duo<R> cw[CX * CY], z0[WX2 * WY2], r1[WX1 * WY1], z1[WX1 * WY1];
+  __shared__ C di[WX1 * WY1];
+  const int N = L.N, nn = N * N, Nc = (N - 1) / 2, nnc = Nc * Nc;
+  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, tid = threadIdx.y * TX + threadIdx.x;
+  const C mu = shift_of<R>(tab, 2 * blockIdx.z, kind);
+  const long long o0 = 2LL * blockIdx.z * nn, o1 = o0 + nn;
+  const C* __restrict__ c0 = coarse + 2LL * blockIdx.z * nnc;
+  const C zero = mk<R>(0, 0);
+  for (int e = tid; e < CX * CY; e += 256) {
+    const int lj = e / CX, ci = x0 / 2 - 2 + e - lj * CX, cj = y0 / 2 - 2 + lj;
+    const bool in = ci >= 0 && ci < Nc && cj >= 0 && cj < Nc;
+    cw[e].v[0] = in ? c0[cj * Nc + ci] : zero;
+    cw[e].v[1] = in ? c0[nnc + cj * Nc + ci] : zero;
+  }
+  __syncthreads();
+  for (int e = tid; e < WX2 * WY2; e += 256) {
+    const int lj = e / WX2, li = e - lj * WX2, gi = x0 - 2 + li, gj = y0 - 2 + lj;
+    Duo<R> z{{zero, zero}};
+    if (gi >= 0 && gi < N && gj >= 0 && gj < N) {
+      const int pt = gj * N + gi;
+      // prolong_pt's sum over (Ka|Kb) pairs, from the window
+      const int ia = (li + 1) >> 1, ib = (li + 2) >> 1, ja = ((lj + 1) >> 1) * CX, jb = ((lj + 2) >> 1) * CX;
+      const Duo<R> c11 = cw[ja + ia], c21 = cw[ja + ib], c12 = cw[jb + ia], c22 = cw[jb + ib];
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+        z.v[k] = cadd(zin[(k ? o1 : o0) + pt],
+                      cscale(cadd(cadd(c11.v[k], c21.v[k]), cadd(c12.v[k], c22.v[k])), (R)0.25));
+    }
+    z0[e] = z;
+  }
+  __syncthreads();
+  for (int e = tid; e < WX1 * WY1; e += 256) {
+    const int lj = e / WX1, li = e - lj * WX1, gi = x0 - 1 + li, gj = y0 - 1 + lj, at = (lj + 1) * WX2 + li + 1;
+    Duo<R> r{{zero, zero}}, z{{zero, zero}};
+    C dinv = zero;
+    if (gi >= 0 && gi < N && gj >= 0 && gj < N) {
+      const int pt = gj * N + gi;
+      r.v[0] = rhs[o0 + pt];
+      r.v[1] = rhs[o1 + pt];
+      dinv = jacobi_dinv<R>(L, mu, pt);
+      z = jacobi_win<R, WX2>(L, mu, dinv, r, z0, at, gi, gj, w);
+    }
+    r1[e] = r;
+    di[e] = dinv;
+    z1[e] = z;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int ty = threadIdx.y + 8 * h, gi = x0 + threadIdx.x, gj = y0 + ty;
+    if (gi < N && gj < N) {
+      const int at = (ty + 1) * WX1 + threadIdx.x + 1, pt = gj * N + gi;
+      const Duo<R> z = jacobi_win<R, WX1>(L, mu, di[at], r1[at], z1, at, gi, gj, w);
+      if (base) {
+        base[o0 + pt] = cadd(base[o0 + pt], z.v[0]);
+        base[o1 + pt] = cadd(base[o1 + pt], z.v[1]);
+      } else {
+        zout[o0 + pt] = z.v[0];
+        zout[o1 + pt] = z.v[1];
       }
-      z2[k][e] = v;
-    }
-  }
-  __syncthreads();
-  // the tile: the smoothed solution and its residual
-  const int gi = x0 + threadIdx.x, gj = y0 + threadIdx.y;
-  if (gi < N && gj < N) {
-    const int li1 = threadIdx.x + 1, lj1 = threadIdx.y + 1, pt = gj * N + gi;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const C zc = z2[k][lj1 * WX1 + li1];
-      const C Az = cadd(cmul(mu, zc), tauKz_win<R>(L, z2[k], WX1, li1, lj1, gi, gj));
-      zout[o0 + (long long)k * nn + pt] = zc;
-      res[o0 + (long long)k * nn + pt] = csub(r2[k][(threadIdx.y + 2) * WX2 + threadIdx.x + 2], Az);
     }
   }
 }
@@ -924,9 +1018,10 @@ __global__ void __launch_bounds__((mg_time_threads<R, n>()), (lane::time_blocks_
 // ------------------------------------------------------------------------------------------
 static unsigned blocks_for(long long len) { return (unsigned)((len + 255) / 256); }
 
+// `base`: see k_mg_postsmooth (FP32 Dirichlet levels with a coarser one only)
 template <typename R>
 static void vcycle(const MgHost& h, const cx<R>* tab, int kind, int l, const cx<R>* rhs, cx<R>* z, cx<R>* spare,
-                   cudaStream_t st) {
+                   cudaStream_t st, cx<R>* base = nullptr) {
   const MgLevel& L = h.lev[l];
   if (l > 0 && l == h.tail_l0) {      // the coarse levels in one launch, one block per slot
     MgTail T;
@@ -947,28 +1042,33 @@ static void vcycle(const MgHost& h, const cx<R>* tab, int kind, int l, const cx<
     g_mg_launches += 1;
     return;
   }
+  // FP32 on a Dirichlet level: one launch before the restriction and one after the coarse levels.  Not in
+  // FP64: the fused kernels repeat the sweeps on their halos, and the FP64 rate bounds those (level 0 at
+  // N = 255, n = 256: 2.32 ms fused against about 1.9 ms for the three launches of the pre-smoothing).
+  if constexpr (sizeof(R) == 4 && kNu == 2) {
+    if (!L.neu) {
+      const MgLevel& C = h.lev[l + 1];
+      const dim3 tiles = tile_grid(L.N, h.nsys / 2);
+      k_mg_presmooth<R><<<tiles, kMgBlock, 0, st>>>(L, tab, kind, rhs, spare, z, w);    // solution, residual
+      k_mg_restrict<R, false><<<grid_for(C.N, h.nsys / 2), kMgBlock, 0, st>>>(L.N, z, (cx<R>*)C.a[0]);
+      vcycle<R>(h, tab, kind, l + 1, (cx<R>*)C.a[0], (cx<R>*)C.a[1], (cx<R>*)C.a[2], st);
+      k_mg_postsmooth<R><<<tiles, kMgBlock, 0, st>>>(L, tab, kind, rhs, spare, (const cx<R>*)C.a[1], z, base, w);
+      g_mg_launches += 3;
+      return;
+    }
+  }
   // pre-smoothing from zero: the first sweep z1 = w D^{-1} rhs, then nu1 - 1 sweeps ping-ponging
   // between `spare` and z.  The nu1 + nu2 = 2 nu sweeps alternate between the two buffers, so
   // starting in `spare` leaves the last post-smoothing sweep in z.
   cx<R>* cur = spare;
   cx<R>* oth = z;
-  if (!L.neu && kNu == 2 && sizeof(R) == 4) {
-    // both sweeps and the residual in one launch: the solution in z, the residual in `spare`.
-    // FP32 only: the fused kernel repeats the sweeps on its halos, and in FP64, whose kernels are
-    // bound by the FP64 rate rather than by memory, that costs more than it saves (level 0 at
-    // N = 255, n = 256: 2.32 ms fused against about 1.9 ms for the three launches)
-    k_mg_presmooth<R><<<grids, kMgBlock, 0, st>>>(L, tab, kind, rhs, z, spare, w);
-    cur = z; oth = spare;
-    g_mg_launches += 1;
-  } else {
-    k_mg_jacobi<R, true><<<grids, kMgBlock, 0, st>>>(L, tab, kind, rhs, nullptr, cur, w);
-    for (int s = 1; s < kNu; ++s) {
-      k_mg_jacobi<R, false><<<grids, kMgBlock, 0, st>>>(L, tab, kind, rhs, cur, oth, w);
-      std::swap(cur, oth);
-    }
-    k_mg_resid<R><<<grids, kMgBlock, 0, st>>>(L, tab, kind, rhs, cur, oth);
-    g_mg_launches += kNu + 1;
+  k_mg_jacobi<R, true><<<grids, kMgBlock, 0, st>>>(L, tab, kind, rhs, nullptr, cur, w);
+  for (int s = 1; s < kNu; ++s) {
+    k_mg_jacobi<R, false><<<grids, kMgBlock, 0, st>>>(L, tab, kind, rhs, cur, oth, w);
+    std::swap(cur, oth);
   }
+  k_mg_resid<R><<<grids, kMgBlock, 0, st>>>(L, tab, kind, rhs, cur, oth);
+  g_mg_launches += kNu + 1;
   // restrict the residual to the coarse right-hand side
   const MgLevel& C = h.lev[l + 1];
   const dim3 gridc = grid_for(C.N, h.nsys / 2);
@@ -1016,9 +1116,10 @@ static cudaError_t mg_apply(const Batch& B, const Geom& g, const MgHost& h, int 
       vcycle<R>(h, tab, kind, 0, r0, z0, (T*)F.a[1], st);
     } else {
       k_mg_resid<R><<<grid_for(F.N, h.nsys / 2), kMgBlock, 0, st>>>(F, tab, kind, r0, z0, x0);
-      vcycle<R>(h, tab, kind, 0, x0, (T*)F.a[2], (T*)F.a[1], st);
-      k_mg_axpy<R><<<blocks_for(len), 256, 0, st>>>(len, (const T*)F.a[2], z0, 0);
-      g_mg_launches += 2;
+      const bool adds = sizeof(R) == 4 && !F.neu && h.nlev > 1;   // the last kernel of the cycle adds to z0
+      vcycle<R>(h, tab, kind, 0, x0, (T*)F.a[2], (T*)F.a[1], st, adds ? z0 : nullptr);
+      if (!adds) k_mg_axpy<R><<<blocks_for(len), 256, 0, st>>>(len, (const T*)F.a[2], z0, 0);
+      g_mg_launches += 1 + !adds;
     }
   }
   k_mg_time_inv<R, n><<<tb, threads, smem, st>>>(B.G, B.S, out_slot, tab, kind, z0);
