@@ -33,7 +33,7 @@ sys.path.insert(0, ROOT)
 WORKLOAD = dict(name="heat-control N=511 n=512 backward-Euler a=1 (2.67e8 unknowns), gamma {1e-2,1e-6}",
                 N=511, n=512, theta=1.0, T=1.0, gammas=(1e-2, 1e-6))
 METRIC = "solves/s to relres 1e-8 (mixed-precision MINRES-|P_S|)"
-PROFILE_TRAFFIC = os.path.join(ROOT, "profiles", "precond_apply_N511_n512.md")
+PROFILE_TRAFFIC = os.path.join(ROOT, "profiles", "precond_lane_N511_n512.md")
 # FP64 instructions per output value of the theta = 1 FP64 product with an epilogue (true
 # residuals): the epilogue's scale folded into the operator's coefficients, ten operations
 MV_FP64_OPS = 10.0
@@ -208,7 +208,7 @@ def profile_traffic():
             if line.startswith("traffic_bytes_per_apply:"):
                 traffic = float(line.split(":", 1)[1].strip())
         h = hashlib.sha256()
-        for f in ("fft_reg.cuh", "precond.cu", "precond_pipe.cu", "pcb_internal.cuh"):
+        for f in ("f32_convert.cuh", "fft_reg.cuh", "precond_lane.cuh", "pcb_internal.cuh"):
             h.update(open(os.path.join(ROOT, "paper_2406_00952_gb300", "csrc", f), "rb").read())
         return traffic if (want == h.hexdigest() and traffic) else None
     except Exception:

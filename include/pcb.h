@@ -96,8 +96,7 @@ typedef struct {
   double T;               /* horizon, > 0                                                      */
   double gamma;           /* regularisation, > 0                                               */
   double zeta;            /* omega = exp(i zeta), Sec. 2 (pi: the paper's skew-circulant).      */
-                          /* Any zeta runs the pipelined FP32 kernels for n <= 512 (pi also for */
-                          /* n = 1024); variable a(x) needs zeta = pi                           */
+                          /* Any zeta runs the same kernels; variable a(x) needs zeta = pi      */
   const double* a_edges;  /* host; NULL => a(x) = 1; else 2*N*(N+1) values of a at cell-edge   */
                           /* midpoints: first ax[j][e] (N rows of N+1; x1-edge between nodes   */
                           /* e and e+1 of row j+1), then ay[e][i] (N+1 rows of N)              */
@@ -170,10 +169,10 @@ int pcb_precond_apply(pcb_problem* p, int kind, int precision, const double* x_d
 
 /* ---- autotuning of the preconditioner's kernel shapes ------------------------------------ */
 /* The transforms of Sec. 3.5 (steps 1 and 3) can run in several kernel configurations: the
- * pipelined FP32 kernels or the tile kernels for the spatial and the time passes (and, for n = 512,
- * with or without handing the time pass contiguous time lines, and with 2, 3 or 4 resident blocks
- * per SM for that time pass), and for the tile kernels several register-FFT radices (values per
- * lane) and tile sizes.  pcb_autotune times `reps` applications
+ * kernels with one line per lane (the default where the shape has them), the pipelined FP32 kernels
+ * or the tile kernels for the spatial and the time passes (and, for n = 512, with or without handing
+ * the time pass contiguous time lines, and with 2, 3 or 4 resident blocks per SM for that time pass),
+ * and for the tile kernels several register-FFT radices (values per lane) and tile sizes.  pcb_autotune times `reps` applications
  * of preconditioner `kind` (PCB_PREC_NONE: the problem's default) in the problem's precision under
  * each configuration that fits the problem's shape, keeps the fastest for this problem, and records
  * it for the device and shape (N, n, boundary condition, zeta = pi or not, precision): problems
@@ -189,8 +188,8 @@ typedef struct {
   int chosen;              /* index of the winner among them (0: the default configuration)      */
   double default_ms;       /* mean apply time of the default configuration                       */
   double best_ms;          /* mean apply time of the winner                                      */
-  int pipelined_dst;       /* winner: pipelined spatial passes (1) or tile kernels (0)            */
-  int pipelined_time;      /* winner: pipelined time pass (1) or tile kernel (0)                  */
+  int pipelined_dst;       /* winner: pipelined spatial passes (1); 0: one line per lane, or tiles*/
+  int pipelined_time;      /* winner: pipelined time pass (1); 0: one line per lane, or tiles     */
   int time_major_handoff;  /* winner: the n = 512 spatial pass writes contiguous time lines       */
   int dst_lanes;           /* lanes per spatial line of the tile kernels (values per lane = M/lanes)*/
   int time_lanes;          /* lanes per time line of the tile kernels                            */
