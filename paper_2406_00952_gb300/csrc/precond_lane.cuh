@@ -18,11 +18,11 @@
 //
 // What bounds the passes and what they measured (one GB300, ncu durations; in brackets the pipelined
 // kernels of precond_pipe.cu, which remain the alternative a caller can pin, and the tile kernels):
-//   N = 511, n = 512, FP32: pass 1 0.61 ms (0.83), pass 2 0.32 (0.68; 6.5 TB/s, at the HBM limit), time 0.60
-//   (0.83), pass 4 0.35 (0.65; 6.0 TB/s), pass 5 0.65 (0.59); the apply 2.55 ms (3.53).  Passes 1 and 5 wait for
+//   N = 511, n = 512, FP32: pass 1 0.61 ms (0.83), pass 2 0.32 (0.68; 6.5 TB/s, at the HBM limit), time 0.58
+//   (0.83), pass 4 0.35 (0.65; 6.0 TB/s), pass 5 0.65 (0.59); the apply 2.54 ms (3.53).  Passes 1 and 5 wait for
 //   the conversion of their FP64 side between load and store, the time pass for its two barriers with
 //   only 16 warps a multiprocessor (128 registers).
-//   N = 255, n = 256, FP64: spatial passes 1.06 ms each, time 2.2, the apply 6.5 ms (14.7): 89% of the FP64
+//   N = 255, n = 256, FP64: spatial passes 1.06 ms each, time 2.03, the apply 6.3 ms (14.7): 89% of the FP64
 //   issue rate on the operations of the symmetric transform.
 //   N = 383, n = 64, FP32 (tile kernels before): apply 0.21 ms (1.00).
 #pragma once
@@ -555,15 +555,16 @@ __device__ __forceinline__ void solve_pair(int kind, cx<R>& Xr, cx<R>& Xq, cx<R>
   using T = cx<R>;
   if (kind == PK_PS) {
     const T lam = mk<R>(mr.x + c, mr.y);
+    // 20 operations and a division, where forming F1, F2, U1 and U2 takes 30 (with odd_dft: FP64 time pass at
+    // N = 255, n = 256 2.21 -> 2.03 ms): with U1, U2 the solved halves, Xr' = U1 + i U2 and Xq' = conj U1 + i conj U2 collapse to
+    //   Xr' = ((a - i alpha) Xr - i b conj Xq) iv,  Xq' = ((a - i alpha) Xq + i b conj Xr) iv,  lambda = a + i b
     const R iv = scale / (lam.x * lam.x + (lam.y * lam.y + a2));
-    const R hi = (R)0.5 * iv;
-    const T Cq = cconj(Xq);
-    const T F1 = cadd(Xr, Cq);
-    const T F2 = cmul_mi(csub(Xr, Cq));
-    const T U1 = cscale(cadd(cmul(cconj(lam), F1), cscale(F2, alpha)), hi);
-    const T U2 = cscale(csub(cmul(lam, F2), cscale(F1, alpha)), hi);
-    Xr = cadd(U1, cmul_pi(U2));
-    Xq = cadd(cconj(U1), cmul_pi(cconj(U2)));
+    const R a = lam.x * iv, b = lam.y * iv, al = alpha * iv;
+    const T x = Xr, q = Xq;
+    Xr.x = a * x.x + (al * x.y - b * q.y);
+    Xr.y = a * x.y - (al * x.x + b * q.x);
+    Xq.x = a * q.x + (al * q.y + b * x.y);
+    Xq.y = a * q.y - (al * q.x - b * x.x);
     return;
   }
   R w;
@@ -702,12 +703,11 @@ __global__ void __launch_bounds__((TimeShape<R, n>::B == 1 ? 128 : time_threads<
       } else {
 #pragma unroll
         for (int q = 0; q < A; ++q) x[q] = in.get(q * istep);
-#pragma unroll
-        for (int q = 1; q < A; ++q) x[q] = cmul(x[q], root64<R>(q * (32 / A)));
       }
-      reg_dft<T, R, A>(x, false);
+      if constexpr (GZ) reg_dft<T, R, A>(x, false);
+      else odd_dft<T, R, A>(x);
 #pragma unroll
-      for (int k = 0; k < A; ++k) ex[((H - 1) * n + t * A + k) * LT] = x[pos<A>(k)];
+      for (int k = 0; k < A; ++k) ex[((H - 1) * n + t * A + k) * LT] = x[GZ ? pos<A>(k) : k];
     }
     __syncthreads();
     // second step, pointwise solve, inverse second step: rows (k1, A-1-k1), or row k1 of both halves
@@ -765,7 +765,8 @@ __global__ void __launch_bounds__((TimeShape<R, n>::B == 1 ? 128 : time_threads<
       T x[A];
 #pragma unroll
       for (int k = 0; k < A; ++k) x[k] = ex[(t * A + k) * LT];
-      reg_dft<T, R, A>(x, true);
+      if constexpr (GZ) reg_dft<T, R, A>(x, true);
+      else odd_idft<T, R, A>(x);
       if constexpr (GZ) {
         R real[A];
 #pragma unroll
@@ -785,8 +786,7 @@ __global__ void __launch_bounds__((TimeShape<R, n>::B == 1 ? 128 : time_threads<
         }
       } else if (ok) {
 #pragma unroll
-        for (int q = 0; q < A; ++q)
-          out.put(q * ostep, q ? mulc(x[pos<A>(q)], root64<R>(q * (32 / A))) : x[pos<A>(q)]);
+        for (int q = 0; q < A; ++q) out.put(q * ostep, x[q]);
       }
     }
   }
