@@ -6,7 +6,8 @@
 //           classical Gram-Schmidt applied twice, Givens rotations on the Hessenberg column.
 // Reductions are deterministic: each block of an instance writes one partial for a fixed slice
 // of the vector, and one block per instance adds the partials in a fixed order, so a result does
-// not depend on which other instances share the launch.
+// not depend on which other instances share the launch.  (MINRES's r1 . y has two such orders, the vector
+// blocks and the tiles of the fused preconditioner passes; which one holds is decided per instance.)
 #include <math.h>
 
 #include "pcb_internal.cuh"
@@ -40,11 +41,13 @@ __device__ __forceinline__ double block_sum(double v) {
   const long long stride = (long long)g.vec_blocks * blockDim.x;   \
   const long long e0 = (long long)lb * blockDim.x + threadIdx.x;
 
-// partial[blk] = sum a.b over the instance's slice
+// partial[blk] = sum a.b over the instance's slice.  skip (k_axpby too): instances to leave out, or null
 __global__ void __launch_bounds__(256) k_dot(const Geom* __restrict__ G, const Slots* __restrict__ S,
                                              const int* __restrict__ off, int count, const int* __restrict__ active,
-                                             int sa, int sb, double* __restrict__ partial) {
+                                             const int* __restrict__ skip, int sa, int sb,
+                                             double* __restrict__ partial) {
   INST_PROLOGUE
+  if (skip && skip[inst]) return;
   const double* __restrict__ a = S[inst].v[sa];
   const double* __restrict__ b = S[inst].v[sb];
   double acc = 0.0;
@@ -57,8 +60,10 @@ __global__ void __launch_bounds__(256) k_dot(const Geom* __restrict__ G, const S
 enum { AX_COPY = 0, AX_MINRES_R = 1, AX_SCALE_INV_BETA = 2, AX_SCALE_INV_HNORM = 3, AX_ADD = 4, AX_ZERO = 5 };
 __global__ void __launch_bounds__(256) k_axpby(const Geom* __restrict__ G, const Slots* __restrict__ S,
                                                const Scal* __restrict__ Sc, const int* __restrict__ off, int count,
-                                               const int* __restrict__ active, int mode, int sx, int sy, int sz) {
+                                               const int* __restrict__ active, const int* __restrict__ skip, int mode,
+                                               int sx, int sy, int sz) {
   INST_PROLOGUE
+  if (skip && skip[inst]) return;
   const Scal& c = Sc[inst];
   const double* __restrict__ x = sx >= 0 ? S[inst].v[sx] : nullptr;
   double* __restrict__ y = S[inst].v[sy];
@@ -423,15 +428,18 @@ __global__ void __launch_bounds__(32) k_backsub(int count, const int* __restrict
   }
 }
 
-// Sum the instance's partials (one per block) and run a scalar step.
+// Sum the instance's partials (one per block) and run a scalar step.  code2: the instances with a nonzero
+// code have theirs at off2, the others at base + off (null: all at off, base 0).
 __global__ void __launch_bounds__(512) k_reduce(const int* __restrict__ off, int count, const int* __restrict__ active,
                                                 const double* __restrict__ partial, Scal* Sc,
                                                 int step, double tol, const double* __restrict__ tols, int j,
-                                                int restart, Slots* S, int a0, int s0, int a1, int s1) {
+                                                int restart, Slots* S, int a0, int s0, int a1, int s1,
+                                                const int* __restrict__ off2, const int* __restrict__ code2, int base) {
   const int inst = blockIdx.x;
   if (inst >= count) return;
   if (active && !active[inst]) return;
-  const int b0 = off[inst], b1 = off[inst + 1];
+  const bool second = code2 && code2[inst];
+  const int b0 = second ? off2[inst] : base + off[inst], b1 = second ? off2[inst + 1] : base + off[inst + 1];
   // the products leave tens of thousands of partials of a large instance: four loads in flight per thread
   // (N = 511, n = 512: 64 -> 17 us)
   double a4[4] = {0.0, 0.0, 0.0, 0.0};
@@ -501,18 +509,40 @@ __global__ void k_setslot(const Geom* __restrict__ G, Slots* S, int count, const
 // host launchers
 // ------------------------------------------------------------------------------------------
 cudaError_t launch_dot(const Batch& B, int sa, int sb) {
-  k_dot<<<B.tot_vec, 256, 0, B.stream>>>(B.G, B.S, B.off_vec, B.count, B.active, sa, sb, B.partial);
+  k_dot<<<B.tot_vec, 256, 0, B.stream>>>(B.G, B.S, B.off_vec, B.count, B.active, nullptr, sa, sb, B.partial);
+  return cudaGetLastError();
+}
+// the residual update and the inner product of a MINRES batch's instances without the fused passes (code 0);
+// their partials follow those of the fused passes' tiles
+cudaError_t launch_minres_rest_residual(const Batch& B, int q, int r2, int r1) {
+  k_axpby<<<B.tot_vec, 256, 0, B.stream>>>(B.G, B.S, B.Sc, B.off_vec, B.count, B.active, B.lane_sp[1], AX_MINRES_R, q, r2,
+                                           r1);
+  return cudaGetLastError();
+}
+cudaError_t launch_minres_rest_dot(const Batch& B, int sa, int sb) {
+  k_dot<<<B.tot_vec, 256, 0, B.stream>>>(B.G, B.S, B.off_vec, B.count, B.active, B.lane_sp[1], sa, sb,
+                                         B.partial + B.tot_ls[1]);
   return cudaGetLastError();
 }
 cudaError_t launch_reduce(const Batch& B, const int* off, int step, double tol, int j, int restart, int a0, int b0,
                           int a1, int b1) {
   // one block size for every instance: the order of its sum must not depend on the batch it is in
   k_reduce<<<B.count, 512, 0, B.stream>>>(off, B.count, B.active, B.partial, B.Sc, step, tol, B.tols, j, restart,
-                                          B.S, a0, b0, a1, b1);
+                                          B.S, a0, b0, a1, b1, nullptr, nullptr, 0);
+  return cudaGetLastError();
+}
+// MINRES's scalar step after r1 . y: fused = its partials are the tiles of the preconditioner's passes
+// (launch_precond_minres), for the instances that have them
+cudaError_t launch_reduce_minres(const Batch& B, bool fused, double tol, int a0, int b0, int a1, int b1) {
+  if (!fused) return launch_reduce(B, B.off_vec, SS_MINRES_GIVENS, tol, 0, 0, a0, b0, a1, b1);
+  if (B.tot_dst_i[1] == 0) return launch_reduce(B, B.off_ls[1], SS_MINRES_GIVENS, tol, 0, 0, a0, b0, a1, b1);
+  k_reduce<<<B.count, 512, 0, B.stream>>>(B.off_vec, B.count, B.active, B.partial, B.Sc, SS_MINRES_GIVENS, tol, B.tols, 0, 0,
+                                          B.S, a0, b0, a1, b1, B.off_ls[1], B.lane_sp[1], B.tot_ls[1]);
   return cudaGetLastError();
 }
 cudaError_t launch_axpby(const Batch& B, int mode, int sx, int sy, int sz) {
-  k_axpby<<<B.tot_vec, 256, 0, B.stream>>>(B.G, B.S, B.Sc, B.off_vec, B.count, B.active, mode, sx, sy, sz);
+  k_axpby<<<B.tot_vec, 256, 0, B.stream>>>(B.G, B.S, B.Sc, B.off_vec, B.count, B.active, nullptr, mode, sx, sy,
+                                            sz);
   return cudaGetLastError();
 }
 cudaError_t launch_minres_wx(const Batch& B, int sy, int sw, int sw2, int sx) {

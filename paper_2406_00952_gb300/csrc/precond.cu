@@ -785,18 +785,24 @@ static cudaError_t lane_passes(const Batch& B, int kind, int in_slot, int out_sl
   return spatial(5, timed, out_slot);
 }
 
+// the five passes of the instances without one-line-per-lane kernels
 template <typename R>
-static cudaError_t precond_passes(const Batch& B, int kind, int in_slot, int out_slot) {
+static cudaError_t other_passes(const Batch& B, int kind, int in_slot, int out_slot) {
   cudaError_t e;
-  if (B.lane_sp_set[sizeof(R) == 4]) {
-    if ((e = lane_passes<R>(B, kind, in_slot, out_slot)) != cudaSuccess) return e;
-    if (B.tot_dst_i[sizeof(R) == 4] == 0) return cudaSuccess;
-  }
   if ((e = dst_pass<R>(B, 1, in_slot, -1)) != cudaSuccess) return e;
   if ((e = dst_pass<R>(B, 2, -1, -1)) != cudaSuccess) return e;
   if ((e = time_pass<R>(B, kind)) != cudaSuccess) return e;
   if ((e = dst_pass<R>(B, 4, -1, -1)) != cudaSuccess) return e;
   return dst_pass<R>(B, 5, -1, out_slot);
+}
+
+template <typename R>
+static cudaError_t precond_passes(const Batch& B, int kind, int in_slot, int out_slot) {
+  if (B.lane_sp_set[sizeof(R) == 4]) {
+    const cudaError_t e = lane_passes<R>(B, kind, in_slot, out_slot);
+    if (e != cudaSuccess || B.tot_dst_i[sizeof(R) == 4] == 0) return e;
+  }
+  return other_passes<R>(B, kind, in_slot, out_slot);
 }
 
 int precond_launch_count(bool var_a, int kind) { return var_a ? mg_launch_count(kind) : 5; }
@@ -879,15 +885,23 @@ cudaError_t launch_fem_spatial(const Batch& B, int mode, int op, int in_slot, in
 
 // MINRES's residual update, preconditioner and inner product in the five passes: r1 = q + rf r2 (scalars of
 // the instance) to slot r1, y = P^{-1} r1 to slot y, partial[b] = the blocks' sums of r1 . y over B.off_ls[1].
-// *fused = false, and nothing launched, unless every instance takes the one-line-per-lane FP32 passes on
-// a Dirichlet grid.  (B.fuse_z != 0 marks the fused passes: slot 0 is never a Krylov vector.)
+// *fused = false, and nothing launched, unless an instance takes the one-line-per-lane FP32 passes.  Others
+// of the batch (B.tot_dst_i[1] > 0) keep kernels of their own, so that each instance's sum has the same
+// order whatever it shares the launches with: launch_reduce_minres finds both kinds of partials.  (MINRES
+// runs on Dirichlet grids.  B.fuse_z != 0 marks the fused passes: slot 0 is never a Krylov vector.)
+cudaError_t launch_minres_rest_residual(const Batch& B, int q, int r2, int r1);
+cudaError_t launch_minres_rest_dot(const Batch& B, int r1, int y);
 cudaError_t launch_precond_minres(const Batch& B, int kind, int prec, int q, int r2, int r1, int y, bool* fused) {
-  *fused = prec == PCB_MIXED && B.lane_sp_set[1] && B.tot_dst_i[1] == 0 && !(B.lane_sp_set[1] >> 12);
+  *fused = prec == PCB_MIXED && B.lane_sp_set[1] && !(B.lane_sp_set[1] >> 12);
   if (!*fused) return cudaSuccess;
   Batch F = B;
   F.fuse_r2 = r2;
   F.fuse_z = r1;
-  return lane_passes<float>(F, kind, q, y);
+  cudaError_t e = lane_passes<float>(F, kind, q, y);
+  if (e != cudaSuccess || B.tot_dst_i[1] == 0) return e;
+  if ((e = launch_minres_rest_residual(B, q, r2, r1)) != cudaSuccess) return e;
+  if ((e = other_passes<float>(B, kind, r1, y)) != cudaSuccess) return e;
+  return launch_minres_rest_dot(B, r1, y);
 }
 
 // B.dst_q / B.time_q = 0 selects the shared-launch kernels for instances of different sizes.

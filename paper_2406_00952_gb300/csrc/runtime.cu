@@ -56,6 +56,8 @@ cudaError_t launch_dot(const Batch& B, int sa, int sb);
 // a0 >= 0: after the step, exchange the instance's slots a0, b0 and a1, b1
 cudaError_t launch_reduce(const Batch& B, const int* off, int step, double tol, int j, int restart, int a0 = -1,
                           int b0 = -1, int a1 = -1, int b1 = -1);
+cudaError_t launch_reduce_minres(const Batch& B, bool fused, double tol, int a0 = -1, int b0 = -1, int a1 = -1,
+                                 int b1 = -1);
 cudaError_t launch_axpby(const Batch& B, int mode, int sx, int sy, int sz);
 cudaError_t launch_minres_wx(const Batch& B, int sy, int sw, int sw2, int sx);
 cudaError_t launch_minres_wx2(const Batch& B, int sy0, int sy1, int sw, int sw2, int sx);
@@ -823,7 +825,7 @@ static int minres_iter_launches(pcb_problem* p, const Batch& B, const SolveCfg& 
     CK(LC(p) launch_dot(B, SL_R1, s_out));
   }
   // (the scalar step also rotates the slots; y_{k+1} of the update then sits in slot Q)
-  CK(LC(p) launch_reduce(B, fused ? B.off_ls[1] : B.off_vec, SS_MINRES_GIVENS, c.tol, 0, 0, SL_R1, SL_R2, SL_Y, s_out));
+  CK(LC(p) launch_reduce_minres(B, fused, c.tol, SL_R1, SL_R2, SL_Y, s_out));
   if (second) CK(LC(p) launch_minres_wx2(B, SL_YO, SL_Q, SL_W, SL_W2, s_x));
   return PCB_OK;
 }
@@ -1653,7 +1655,7 @@ int group_setup(BGroup& G, const SolveCfg& c, const double* const* b_dev, double
   }
   size_t part = 0; int tv = 0, tm = 0, tl = 0;
   for (const Geom& g : gs) { tv += g.vec_blocks; tm += g.mv_blocks; tl += g.ls_blocks[1]; }
-  part = std::max((size_t)tv * (PCB_MAX_RESTART + 1), (size_t)std::max(tm, tl)) + 1;
+  part = std::max((size_t)tv * (PCB_MAX_RESTART + 1), (size_t)std::max(tm, tl + tv)) + 1;
   if (cudaMalloc(&G.dG, sizeof(Geom) * n) || cudaMalloc(&G.dS, sizeof(Slots) * n) ||
       cudaMalloc(&G.dSc, sizeof(Scal) * n) || cudaMalloc(&G.dAct, sizeof(int) * n) ||
       cudaMalloc(&G.dOff, sizeof(int) * batch_ints(n)) || cudaMalloc(&G.dPart, part * sizeof(double)) ||
@@ -1749,7 +1751,7 @@ int round_step(BGroup& G, const SolveCfg& c) {
         if ((r = apply_precond(p0, Bx, G.kind, G.prec, SL_R1, SL_YO))) return r;
         CK(launch_dot(Bx, SL_R1, SL_YO));
       }
-      CK(launch_reduce(Bx, fused ? Bx.off_ls[1] : Bx.off_vec, SS_MINRES_GIVENS, c.tol, 0, 0));
+      CK(launch_reduce_minres(Bx, fused, c.tol));
       CK(launch_minres_wx(Bx, SL_Y, SL_W, SL_W2, SL_XI));
       CK(launch_swap(Bx, SL_R1, SL_R2, SL_Y, SL_YO, SL_W, SL_W2));
       return PCB_OK;
@@ -2212,7 +2214,7 @@ int srv_group_step(pcb_server* S, SrvGroup& G) {
         if ((rc = precond(SL_R1, SL_YO))) return rc;
         CK(launch_dot(G.B, SL_R1, SL_YO));
       }
-      CK(launch_reduce(G.B, fused ? G.B.off_ls[1] : G.B.off_vec, SS_MINRES_GIVENS, tol, 0, 0));
+      CK(launch_reduce_minres(G.B, fused, tol));
       CK(launch_minres_wx(G.B, SL_Y, SL_W, SL_W2, SL_XI));
       if ((rc = srv_read(G, st))) return rc;
       for (int k = 0; k < G.cap; ++k) {
