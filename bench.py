@@ -640,7 +640,9 @@ def main():
     value = solves / (ms / 1e3)
     hbm, peak_kind = peaks()
     # kernel figures: one more step, untimed, with CUDA events around every preconditioner apply
-    # and product (profiling launches each MINRES iteration directly instead of from its graph)
+    # and product (profiling launches each MINRES iteration directly instead of from its graph, and
+    # keeps the residual update and the inner product out of the preconditioner's passes: the same
+    # iterates, and precond_ms is that of the passes alone)
     p0 = torch.cuda.Event(enable_timing=True); p1 = torch.cuda.Event(enable_timing=True)
     p0.record(stream)
     pinfos = step(profile=True)

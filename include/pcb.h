@@ -240,7 +240,10 @@ typedef struct {
   double seconds;         /* wall time of the call                                             */
   long long launches;     /* CUDA kernel launches the call issued                              */
   int precond_applies;    /* preconditioner applications                                       */
-  double precond_ms;      /* profile != 0: summed device time of the applications              */
+  double precond_ms;      /* profile != 0: summed device time of the applications.  A profiled   */
+                          /* MINRES solve runs the residual update and the inner product beside  */
+                          /* them, where other solves may run both inside the applications' first */
+                          /* and last pass (same values, so the same iterates)                    */
   int matvecs;            /* operator products (Krylov and true-residual)                      */
   double matvec_ms;       /* profile != 0: summed device time of the products                  */
   int matvecs_inner;      /* products of the inner MINRES iterations of a mixed-precision solve */

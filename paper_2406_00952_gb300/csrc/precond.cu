@@ -743,6 +743,7 @@ static cudaError_t time_pass(const Batch& B, int kind) {
 cudaError_t lane_rows_f32(const Batch& B, Sel sel, int M, bool ev, int stage, int in_sel, int out_sel);
 cudaError_t lane_rows_f64(const Batch& B, Sel sel, int M, bool ev, int stage, int in_sel, int out_sel);
 cudaError_t lane_cols_f32(const Batch& B, Sel sel, int M, bool ev, int stage, int in_sel, int out_sel);
+cudaError_t lane_dot_f32(const Batch& B, Sel sel, int M, int sy, int sz);
 cudaError_t lane_cols_f64(const Batch& B, Sel sel, int M, bool ev, int stage, int in_sel, int out_sel);
 cudaError_t lane_time_f32(const Batch& B, Sel sel, int n, bool gz, int kind, int in_sel, int out_sel);
 cudaError_t lane_time_f64(const Batch& B, Sel sel, int n, bool gz, int kind, int in_sel, int out_sel);
@@ -902,6 +903,15 @@ cudaError_t launch_precond_minres(const Batch& B, int kind, int prec, int q, int
   if ((e = launch_minres_rest_residual(B, q, r2, r1)) != cudaSuccess) return e;
   if ((e = other_passes<float>(B, kind, r1, y)) != cudaSuccess) return e;
   return launch_minres_rest_dot(B, r1, y);
+}
+
+// The inner product r1 . y of a single problem in the order of the fused passes, after a preconditioner apply
+// of its own.  *tiles = false, and nothing launched, where launch_precond_minres would not fuse.
+cudaError_t launch_minres_tile_dot(const Batch& B, int prec, int r1, int y, bool* tiles) {
+  *tiles = prec == PCB_MIXED && B.count == 1 && B.lane_sp_set[1] && !(B.lane_sp_set[1] >> 12);
+  if (!*tiles) return cudaSuccess;
+  const int code = __builtin_ctz(B.lane_sp_set[1]);
+  return lane_dot_f32(B, Sel{B.active, nullptr, code}, kLaneLengths[code - 1], y, r1);
 }
 
 // B.dst_q / B.time_q = 0 selects the shared-launch kernels for instances of different sizes.

@@ -353,6 +353,22 @@ constexpr size_t cols_smem() {
   return rows > spatial_smem<R, M>() ? rows : spatial_smem<R, M>();
 }
 
+// partial[block] = the sum of the block's dots.  Sixteen lanes at a time: the last warp of a block may be half a
+// warp.
+template <int NT>
+__device__ __forceinline__ void tile_sum(double dot, double* __restrict__ partial) {
+  __shared__ double red[NT / 16];
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) dot += __shfl_xor_sync(threadIdx.x & 16 ? 0xffff0000u : 0x0000ffffu, dot, o, 16);
+  if (threadIdx.x % 16 == 0) red[threadIdx.x / 16] = dot;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double sum = 0.0;
+    for (int k = 0; k < NT / 16; ++k) sum += red[k];
+    partial[blockIdx.x] = sum;
+  }
+}
+
 template <typename R, int M, bool EV, bool USER, bool FUSE>
 __global__ void __launch_bounds__(spatial_threads<R, M>(), spatial_blocks<R, M>())
     k_lane_cols(const Geom* __restrict__ G, const Slots* __restrict__ S, const int* __restrict__ off, int count, Sel sel,
@@ -479,20 +495,31 @@ __global__ void __launch_bounds__(spatial_threads<R, M>(), spatial_blocks<R, M>(
         if constexpr (FUSE) dot = fma(b, z0[v.hs + p * rs], fma(a, z0[p * rs], dot));
       }
     }
-    if constexpr (FUSE) {
-      // sixteen lanes at a time: the last warp of a block may be half a warp
-      __shared__ double red[NT / 16];
-#pragma unroll
-      for (int o = 8; o > 0; o >>= 1) dot += __shfl_xor_sync(threadIdx.x & 16 ? 0xffff0000u : 0x0000ffffu, dot, o, 16);
-      if (threadIdx.x % 16 == 0) red[threadIdx.x / 16] = dot;
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        double sum = 0.0;
-        for (int k = 0; k < NT / 16; ++k) sum += red[k];
-        fuse.partial[blockIdx.x] = sum;
-      }
-    }
+    if constexpr (FUSE) tile_sum<NT>(dot, fuse.partial);
   }
+}
+
+// The inner product of the fused pass on its own, tile by tile and value by value in the same order: for
+// solves whose preconditioner is timed alone (profile), so that timing does not change the iterates.
+template <int M>
+__global__ void __launch_bounds__(spatial_threads<float, M>())
+    k_lane_dot(const Geom* __restrict__ G, const Slots* __restrict__ S, const int* __restrict__ off, int count, Sel sel,
+               int sy, int sz, double* __restrict__ partial) {
+  constexpr int NG = Shape<M>::GROUPS, LT = spatial_lanes<float, M>(), N = M / 2 - 1, nb = (N + LT - 1) / LT;
+  const int inst = find_inst(off, count, blockIdx.x);
+  if (sel.skip(inst)) return;
+  const Geom& g = G[inst];
+  const int lt = blockIdx.x - (count > 1 ? __ldg(off + inst) : 0);
+  const int ts = lt / nb, r0 = (lt - ts * nb) * LT;
+  const int l = threadIdx.x % LT, grp = threadIdx.x / LT;
+  double dot = 0.0;
+  if (r0 + l < N) {
+    const long long at0 = (long long)ts * g.m + r0 + l;
+    const double* __restrict__ y = S[inst].v[sy] + at0;
+    const double* __restrict__ z = S[inst].v[sz] + at0;
+    for (int p = grp; p < N; p += NG) dot = fma(y[g.mn + p * N], z[g.mn + p * N], fma(y[p * N], z[p * N], dot));
+  }
+  tile_sum<spatial_threads<float, M>()>(dot, partial);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -21,6 +21,7 @@ namespace pcb {
 // launchers defined in the other translation units
 cudaError_t launch_precond_fast(const Batch& B, int kind, int prec, int in_slot, int out_slot);
 cudaError_t launch_precond_minres(const Batch& B, int kind, int prec, int q, int r2, int r1, int y, bool* fused);
+cudaError_t launch_minres_tile_dot(const Batch& B, int prec, int r1, int y, bool* tiles);
 cudaError_t launch_precond_mg(const Batch& B, const Geom& g, int kind, int prec, int cycles, int in_slot,
                               int out_slot);
 void mg_release(const void* ws);
@@ -812,7 +813,7 @@ static int minres_iter_launches(pcb_problem* p, const Batch& B, const SolveCfg& 
   CK(P_matvec(p, B, PCB_OP_A, SL_Y, SL_Q, SL_R1, EPI_MINRES | (c.prec == PCB_MIXED ? EPI_FAST : 0)));
   CK(LC(p) launch_reduce(B, B.off_mv, SS_MINRES_ALFA, c.tol, 0, 0));
   // residual update, preconditioner and inner product: in the preconditioner's own passes where it can be
-  // (a profiled solve times the preconditioner, so it keeps them apart)
+  // (a profiled solve times the preconditioner alone, so it keeps them apart: the same values in the same order)
   bool fused = false;
   if (!p->prof && c.kind != PCB_PREC_NONE && !p->g.mg_route)
     CK(launch_precond_minres(B, c.kind, c.prec, SL_Q, SL_R2, SL_R1, s_out, &fused));
@@ -822,7 +823,9 @@ static int minres_iter_launches(pcb_problem* p, const Batch& B, const SolveCfg& 
   } else {
     CK(LC(p) launch_axpby(B, AX_MINRES_R, SL_Q, SL_R2, SL_R1));
     if ((rc = P_precond(p, B, c.kind, c.prec, SL_R1, s_out))) return rc;
-    CK(LC(p) launch_dot(B, SL_R1, s_out));
+    if (p->prof && c.kind != PCB_PREC_NONE) CK(launch_minres_tile_dot(B, c.prec, SL_R1, s_out, &fused));
+    if (!fused) CK(launch_dot(B, SL_R1, s_out));
+    p->launches += 1;
   }
   // (the scalar step also rotates the slots; y_{k+1} of the update then sits in slot Q)
   CK(LC(p) launch_reduce_minres(B, fused, c.tol, SL_R1, SL_R2, SL_Y, s_out));
