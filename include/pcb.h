@@ -200,7 +200,9 @@ int pcb_autotune(pcb_problem* p, int kind, int reps, pcb_tune_info* info);
 
 /* Run this problem (only; nothing is recorded for its shape) in configuration `candidate` of the
  * list pcb_autotune times for its shape and precision, in that list's order (0: the default
- * configuration), without timing it; candidate < 0 changes nothing.  `info` (may be NULL) receives
+ * configuration; from 1 on the pipelined and tile kernels in an order that does not change; last, where
+ * the default has one line per lane, the pipelined or tile kernels in their own default shapes), without
+ * timing it; candidate < 0 changes nothing.  `info` (may be NULL) receives
  * the configuration the problem then runs, with `candidates` the length of the list, `chosen` =
  * candidate and zero times.  Lets a caller pin a configuration, and a test compare every one with
  * the oracle.  Errors: INVALID_ARG (candidate past the list), UNSUPPORTED (variable a(x)), CUDA. */

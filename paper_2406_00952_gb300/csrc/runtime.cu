@@ -1330,10 +1330,11 @@ std::vector<TuneChoice> tune_candidates(const Geom& g, int prec) {
     if (tune_valid(g, c, prec)) out.push_back(c);
   };
   add(0, q0d, q0t);                                   // the default shapes come first
-  // then the other kernels' shapes, without the one-line-per-lane passes where the default takes them
+  // then the other kernels' shapes, without the one-line-per-lane passes where the default takes them.  Their
+  // order is fixed, since callers pin by index; the pipelined and tile kernels' own default shapes, which
+  // stood first before there were one-line-per-lane passes, come last.
   Geom d = g;
   const int nl = [&] { Geom t = g; apply_choice(t, TuneChoice{0, q0d, q0t}); return t.lane_sp[prec == PCB_MIXED] ? TUNE_NO_LANE : 0; }();
-  if (nl) add(nl, q0d, q0t);
   apply_choice(d, TuneChoice{nl, q0d, q0t});
   const bool mixed = prec == PCB_MIXED;
   const bool can_pipe_t = mixed && pipe_time_p(d), can_pipe_d = mixed && pipe_dst_p(d);
@@ -1351,6 +1352,7 @@ std::vector<TuneChoice> tune_candidates(const Geom& g, int prec) {
       for (int tq : qt) add(nl | TUNE_NO_PIPE_DST | TUNE_NO_PIPE_TIME | bs, dq, tq);   // tile kernels only
     }
   }
+  if (nl) add(nl, q0d, q0t);
   return out;
 }
 
