@@ -125,16 +125,20 @@ void matvec_shape(Geom& g) {
 }
 
 // theta < 1 (HALF: theta = 1/2), one role of one block of columns: T x1 - alpha x2 marching forward in
-// time (role 0) or alpha x1 + T^T x2 marching backward (role 1).  With u the marched half, the recurrence
-// z_t = (u_t - (1-theta) z_{t-1})/theta gives (B_n u)_t = z_t - z_{t-1} = (u_t - z_{t-1})/theta, so
-//     out = (1/theta + diagonal) u_t - z_{t-1}/theta - (off-diagonal sum) -/+ alpha (other half)
-// and, for theta = 1/2, z_t = 2 u_t - z_{t-1}: eight FP64 operations per value for a constant
-// coefficient (ten when the difference z_t - z_{t-1} and the stencil are formed on their own).  HALF is a
-// template argument because a choice at run time computes both forms of z.  The kernel is bound by
-// FP64 issue: N = 255, n = 256 0.84 -> 0.57 ms, 90% of the measured FP64 rate.
+// time (role 0) or alpha x1 + T^T x2 marching backward (role 1).  With u the marched half and the recurrence
+// z_t = (u_t - (1-theta) z_{t-1})/theta, z_t = 2 u_t - z_{t-1} for theta = 1/2,
+//     out = (z_t - z_{t-1}) + c (4 u_t - sum of neighbours) -/+ alpha (other half),
+// eight FP64 operations per value for theta = 1/2, with a variable coefficient too (ten when each term is
+// rounded on its own).  The order keeps the rounding error at or below that of the separate terms: 4 u - sum
+// is one FMA, c is not added to the coefficient of z (a rounded diagonal 1/theta + 4c, at as many operations,
+// made the error a tenth to a third larger), and a variable coefficient's neighbours, smaller than its
+// diagonal, come before it.  For other theta, whose z has less rounding error of its own, the
+// variable stencil is summed apart.  HALF is a template argument because a choice at run time computes both
+// forms of z.  The kernel is bound by FP64 issue: N = 255, n = 256 0.84 -> 0.57 ms, 90% of the measured FP64
+// rate (variable coefficient 0.95 -> 0.53).
 // A small grid has too few columns to fill the device with one thread each.  Its time range is split
 // in g.mv_chunks parts: a first sweep marches every part from z = 0, the carries combine through
-// (-(1-theta)/theta)^length, and the second sweep computes the values (GMRES
+// r^length, r = -(1-theta)/theta, and the second sweep computes the values (GMRES
 // solve at N = 63, n = 64: 2.71 -> 2.28 ms, its products having taken 84 us each).
 template <bool VAR, bool HALF>
 __device__ __forceinline__ double march_block(const Geom& g, int lb, int op, const double* __restrict__ x,
@@ -149,18 +153,18 @@ __device__ __forceinline__ double march_block(const Geom& g, int lb, int op, con
   const int len = n / chunks, s0 = ch * len;               // n and chunks are powers of two
   const int t0 = role ? n - 1 - s0 : s0;
   const long long step = role ? -(long long)m : m;
-  const double th = g.theta, ith = 1.0 / th, r = (1.0 - th) * ith;
+  const double th = g.theta, ith = 1.0 / th, om = 1.0 - th;
   const long long at0 = (long long)t0 * m + (ok ? col : 0);
   const double* __restrict__ u = x + (role ? mn : 0) + at0;
   double z = 0.0;
   if (chunks > 1) {
     const double* v = u;
     if (ok)
-      for (int k = 0; k < len; ++k, v += step) z = HALF ? fma(ith, *v, -z) : fma(-r, z, ith * *v);
+      for (int k = 0; k < len; ++k, v += step) z = HALF ? fma(2.0, *v, -z) : fma(-om, z, *v) * ith;
     carry[threadIdx.x] = z;
     __syncthreads();
     double pw = 1.0;
-    for (int k = 0; k < len; ++k) pw *= -r;
+    for (int k = 0; k < len; ++k) pw *= -om * ith;
     z = 0.0;
     for (int c = 0; c < ch; ++c) z = fma(pw, z, carry[c * cpb + cl]);
   }
@@ -172,14 +176,12 @@ __device__ __forceinline__ double march_block(const Geom& g, int lb, int op, con
   const int oL = i > 0 ? -1 : (neu ? 1 : 0), oR = i < N - 1 ? 1 : (neu ? -1 : 0);
   const int oD = j > 0 ? -N : (neu ? N : 0), oU = j < N - 1 ? N : (neu ? -N : 0);
   const double alpha = role ? g.alpha : -g.alpha;
-  double kc, kL = 0.0, kR = 0.0, kD = 0.0, kU = 0.0;
+  double kc = 0.0, kL = 0.0, kR = 0.0, kD = 0.0, kU = 0.0;
   if (VAR) {
     const double* ax = g.axs + (long long)j * (N + 1) + i;
     kL = oL ? -ax[0] : 0.0; kR = oR ? -ax[1] : 0.0;
     kD = oD ? -g.ays[col] : 0.0; kU = oU ? -g.ays[col + N] : 0.0;
-    kc = ith + g.dgs[col];
-  } else {
-    kc = fma(4.0, g.c, ith);
+    kc = g.dgs[col];
   }
   const long long offs = (role == 0) == (op == PCB_OP_A) ? mn : 0;
   const double* __restrict__ w = x + (role ? 0 : mn) + at0;
@@ -188,18 +190,21 @@ __device__ __forceinline__ double march_block(const Geom& g, int lb, int op, con
   for (int k = 0; k < len; ++k, u += step, w += step, a += step) {
     const double uc = *u;
     const double l = oL ? u[oL] : 0.0, rr = oR ? u[oR] : 0.0, d = oD ? u[oD] : 0.0, t = oU ? u[oU] : 0.0;
-    double o;
-    if (VAR) {
-      o = fma(kL, l, kc * uc);
+    const double zn = HALF ? fma(2.0, uc, -z) : fma(-om, z, uc) * ith;
+    double o = zn - z;
+    if (VAR && !HALF) {
+      o += fma(kc, uc, fma(kU, t, fma(kD, d, fma(kR, rr, kL * l))));
+    } else if (VAR) {
+      o = fma(kL, l, o);
       o = fma(kR, rr, o);
       o = fma(kD, d, o);
       o = fma(kU, t, o);
+      o = fma(kc, uc, o);
     } else {
-      o = fma(-g.c, (l + rr) + (d + t), kc * uc);
+      o = fma(g.c, fma(4.0, uc, -((l + rr) + (d + t))), o);
     }
-    o = fma(-ith, z, o);
     o = fma(alpha, *w, o);
-    z = HALF ? fma(ith, uc, -z) : fma(-r, z, ith * uc);
+    z = zn;
     out[a] = epi_apply(e, o, aux, x, a, part);
   }
   return part;
