@@ -114,11 +114,14 @@ void matvec_shape(Geom& g) {
     g.mv_blocks = units * ((g.n + tch - 1) / tch);
   } else {
     g.mv_tchunk = g.n;
-    // march_block: parts of the time range while that leaves at least four steps each and the device
-    // short of threads (about 250 a multiprocessor, half of what it holds at this register count; with
-    // more columns the extra operation of the first sweep costs more than the threads give)
+    // march_block: parts of the time range while that leaves at least four steps each and the columns give
+    // the device fewer than about 200 threads a multiprocessor.  The first sweep costs one or two operations
+    // a value and a read of the half; more threads than that no longer pay for it.  n = 128, theta = 1/2
+    // and 0.7, us with 1, 2, 4, 8 parts: N = 63 73, 46, 35, 35 and 76, 52, 41, 42 (4 taken); N = 95 73, 56,
+    // 56, 57 and 77, 68, 69, 72 (2); N = 127 87, 99, 87, 89 and 95, 124, 111, 115 (1); N = 191 167, 204,
+    // 183, 183 and 184, 239, 238, 240 (1).
     g.mv_chunks = 1;
-    while (g.mv_chunks < 8 && g.n / (2 * g.mv_chunks) >= 4 && 2LL * g.m * g.mv_chunks < 76000) g.mv_chunks *= 2;
+    while (g.mv_chunks < 8 && g.n / (2 * g.mv_chunks) >= 4 && 2LL * g.m * g.mv_chunks < 31000) g.mv_chunks *= 2;
     const int cpb = kMvThreads / g.mv_chunks;
     g.mv_blocks = 2 * ((g.m + cpb - 1) / cpb);
   }
