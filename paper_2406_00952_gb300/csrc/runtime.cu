@@ -2017,11 +2017,12 @@ struct SrvLayout {
 
 size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
 
-void srv_layout(const Geom& g, int method, int restart, SrvLayout& L) {
+// (the padded layout of the preconditioner scratch is that of the FP32 passes)
+void srv_layout(const Geom& g, int method, int prec, int restart, SrvLayout& L) {
   const size_t vb = (size_t)2 * g.mn * sizeof(double);
   size_t o = 0;
   L.tab = o; o += up256(table_layout(g, L.tl));
-  L.scr = o; o += up256(std::max<size_t>(vb, (size_t)16 * g.n * g.N * (size_t)g.lr));
+  L.scr = o; o += up256(std::max<size_t>(vb, prec == PCB_MIXED ? (size_t)16 * g.n * g.N * (size_t)g.lr : 0));
   L.minres = o; o += 7 * vb;
   L.mixed = o; o += 2 * vb;
   L.gmres = o; o += method == PCB_MINRES ? 0 : (size_t)(2 * restart + 2) * vb;
@@ -2080,7 +2081,7 @@ long long srv_bytes(const pcb_desc* d, int restart) {
   init_geom(d, g);
   apply_cached_tuning(g, d->precision);
   SrvLayout L;
-  srv_layout(g, srv_method(*d), restart, L);
+  srv_layout(g, srv_method(*d), d->precision, restart, L);
   return (long long)L.total;
 }
 
@@ -2378,7 +2379,7 @@ int srv_admit(pcb_server* S, SrvGroup& G, int k, const SrvReq& r, bool* fitted) 
   init_geom(&r.desc, g);
   apply_cached_tuning(g, S->o.precision);
   SrvLayout L;
-  srv_layout(g, G.method, S->o.restart, L);
+  srv_layout(g, G.method, S->o.precision, S->o.restart, L);
   unsigned char* blk = (unsigned char*)S->arena.alloc(L.total);
   if (!blk) return PCB_OK;
   *fitted = true;
