@@ -1,12 +1,4 @@
-// Register / warp-shuffle FFTs for lines of length M = P * Q (P lanes of a warp, Q values per lane).
-//
-// Lane t of a P-lane group holds x[t + P q], q = 0..Q-1 (consecutive lanes hold consecutive
-// elements, so loads from a contiguous line are conflict-free).  With s = t + P q and
-// k = k1 + Q k2:
-//     X[k1 + Q k2] = sum_t W_P^{t k2} W_M^{t k1} sum_q x[t + P q] W_Q^{q k1}
-// so each lane runs a Q-point DFT in registers, multiplies by W_M^{t k1}, and the P-point DFTs
-// over t run as radix-2 decimation-in-frequency stages across lanes (__shfl_xor), leaving
-// lane t with X[k1 + Q bitrev_P(t)].  Forward uses W = exp(-2 pi i / M); inverse conjugates.
+// Register DFTs: one thread holds the whole sequence.  Forward uses W = exp(-2 pi i / Q); inverse conjugates.
 #pragma once
 #include <math.h>
 
@@ -14,32 +6,8 @@
 
 namespace pcb {
 
-// W_96^k = exp(-2 pi i k / 96): covers every twiddle of the register DFTs (Q | 96) and of the
-// cross-lane stages (2d | 32).  One copy per translation unit that includes this header; each
-// such unit fills its copy with upload_w96() before its first launch.
-static __constant__ float2 c_w96f[96];
-static __constant__ double2 c_w96d[96];
-
-static cudaError_t upload_w96() {
-  float2 f[96];
-  double2 d[96];
-  for (int k = 0; k < 96; ++k) {
-    const double a = -2.0 * 3.14159265358979323846 * k / 96.0;
-    d[k].x = cos(a); d[k].y = sin(a);
-    f[k].x = (float)d[k].x; f[k].y = (float)d[k].y;
-  }
-  cudaError_t e = cudaMemcpyToSymbol(c_w96f, f, sizeof(f));
-  if (e != cudaSuccess) return e;
-  return cudaMemcpyToSymbol(c_w96d, d, sizeof(d));
-}
-
-template <typename R> __device__ __forceinline__ cx<R> w96(int k);
-template <> __device__ __forceinline__ float2 w96<float>(int k) { return c_w96f[k]; }
-template <> __device__ __forceinline__ double2 w96<double>(int k) { return c_w96d[k]; }
-
-// The same roots with a compile-time index (the unrolled register DFTs): cos(2 pi k / 96), k = 0 .. 24,
-// rounded to FP64, and the octant symmetries.  They fold into the instructions, so a unit that uses the
-// register DFTs alone needs no table upload.
+// exp(-2 pi i k / 96), every root of the register DFTs (Q | 96), with a compile-time index: cos(2 pi k / 96),
+// k = 0 .. 24, rounded to FP64, and the octant symmetries.  They fold into the instructions.
 __device__ __forceinline__ constexpr double cos96(int k) {
   constexpr double c[25] = {
     1.0, 0.9978589232386035, 0.9914448613738104, 0.9807852804032304,
@@ -223,60 +191,5 @@ __device__ __forceinline__ void odd_idft(T* x) {
     x[q + H] = cmul_pi(csub(a, b));
   }
 }
-
-// Cross-lane radix-2 DIF over P lanes (P a power of two <= 32) for each of the Q registers.
-// Stage s (half-width d = P >> (s+1)): lower lanes keep v + u, upper lanes (u - v) W_{2d}^{t mod d}.
-// Written as (u + sg*v) * we with sg = +-1 and we = 1 or the twiddle, so every lane runs the
-// same instruction stream (no select).
-template <typename T, typename R>
-struct LaneStages {
-  T we[5];
-  R sg[5];
-  int n;
-};
-
-template <typename T, typename R>
-__device__ __forceinline__ void lane_stages(LaneStages<T, R>& st, int t, int P, bool inv) {
-  const int nst = __ffs(P) - 1;   // log2 P
-#pragma unroll
-  for (int s = 0; s < 5; ++s) {
-    st.we[s] = mk<R>((R)1, (R)0);
-    st.sg[s] = (R)1;
-    if (s < nst) {
-      const int d = P >> (s + 1);
-      const bool upper = (t & d) != 0;
-      T w = w96<R>(((t & (d - 1)) * (96 / (2 * d))) % 96);
-      if (inv) w.y = -w.y;
-      if (upper) { st.we[s] = w; st.sg[s] = (R)-1; }
-    }
-  }
-  st.n = nst;
-}
-
-template <typename T, typename R, int Q>
-__device__ __forceinline__ void lane_dif(T* x, int P, const LaneStages<T, R>& st) {
-#pragma unroll
-  for (int s = 0; s < 5; ++s) {
-    if (s >= st.n) break;
-    const int d = P >> (s + 1);
-    const T w = st.we[s];
-    const R sg = st.sg[s];
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const T v = x[q];
-      T a;
-      a.x = __shfl_xor_sync(0xffffffffu, v.x, d);
-      a.y = __shfl_xor_sync(0xffffffffu, v.y, d);
-      x[q] = cmul(cfma_s(sg, v, a), w);
-    }
-  }
-}
-
-__device__ __forceinline__ int bitrev(int t, int P) {
-  return P <= 1 ? 0 : (int)(__brev((unsigned)t) >> (32 - __ffs(P) + 1));
-}
-
-// padded shared-memory index: one gap every 32 elements
-__device__ __forceinline__ int pidx(int s) { return s + (s >> 5); }
 
 }  // namespace pcb

@@ -144,9 +144,6 @@ static void mg_slot_tables(const Geom& g, MgHost& h, unsigned char*& p);
 static int tail_level(const MgHost& h);
 
 cudaError_t mg_setup(Geom& g, void* ws, const double* a_edges, double a0) {
-  // this translation unit's copy of the register-FFT twiddle table
-  cudaError_t e0 = upload_w96();
-  if (e0 != cudaSuccess) return e0;
   MgHost h;
   const bool neu = g.bc == PCB_BC_NEUMANN;
   h.nlev = levels_for(g.N, neu);

@@ -17,7 +17,7 @@
 //
 // Each pass stages a tile of lines through padded shared memory (coalesced global access in both
 // directions); each line is transformed by a group of P <= 32 lanes holding Q values each
-// (register DFT + warp-shuffle stages, fft_reg.cuh).
+// (register DFT + warp-shuffle stages, below).
 #include <algorithm>
 
 #include "fft_reg.cuh"
@@ -26,6 +26,91 @@ namespace pcb {
 
 enum { PK_ABS_PS = 1, PK_PS = 2, PK_PMS = 3 };
 int mg_launch_count(int kind);
+
+// Lines of length M = P Q over P lanes of a warp, Q values per lane.  Lane t of a P-lane group holds
+// x[t + P q], q = 0..Q-1 (consecutive lanes hold consecutive elements, so loads from a contiguous line
+// are conflict-free).  With s = t + P q and k = k1 + Q k2:
+//     X[k1 + Q k2] = sum_t W_P^{t k2} W_M^{t k1} sum_q x[t + P q] W_Q^{q k1}
+// so each lane runs a Q-point DFT in registers (fft_reg.cuh), multiplies by W_M^{t k1}, and the P-point
+// DFTs over t run as radix-2 decimation-in-frequency stages across lanes (__shfl_xor), leaving lane t
+// with X[k1 + Q bitrev_P(t)].
+//
+// W_96^k = exp(-2 pi i k / 96): the twiddles of the cross-lane stages (2d | 32), whose index depends on the
+// lane.  upload_constants() fills the table before the first launch on a device.
+static __constant__ float2 c_w96f[96];
+static __constant__ double2 c_w96d[96];
+
+cudaError_t upload_constants() {
+  float2 f[96];
+  double2 d[96];
+  for (int k = 0; k < 96; ++k) {
+    const double a = -2.0 * 3.14159265358979323846 * k / 96.0;
+    d[k].x = cos(a); d[k].y = sin(a);
+    f[k].x = (float)d[k].x; f[k].y = (float)d[k].y;
+  }
+  cudaError_t e = cudaMemcpyToSymbol(c_w96f, f, sizeof(f));
+  if (e != cudaSuccess) return e;
+  return cudaMemcpyToSymbol(c_w96d, d, sizeof(d));
+}
+
+template <typename R> __device__ __forceinline__ cx<R> w96(int k);
+template <> __device__ __forceinline__ float2 w96<float>(int k) { return c_w96f[k]; }
+template <> __device__ __forceinline__ double2 w96<double>(int k) { return c_w96d[k]; }
+
+// Cross-lane radix-2 DIF over P lanes (P a power of two <= 32) for each of the Q registers.
+// Stage s (half-width d = P >> (s+1)): lower lanes keep v + u, upper lanes (u - v) W_{2d}^{t mod d}.
+// Written as (u + sg*v) * we with sg = +-1 and we = 1 or the twiddle, so every lane runs the
+// same instruction stream (no select).
+template <typename T, typename R>
+struct LaneStages {
+  T we[5];
+  R sg[5];
+  int n;
+};
+
+template <typename T, typename R>
+__device__ __forceinline__ void lane_stages(LaneStages<T, R>& st, int t, int P, bool inv) {
+  const int nst = __ffs(P) - 1;   // log2 P
+#pragma unroll
+  for (int s = 0; s < 5; ++s) {
+    st.we[s] = mk<R>((R)1, (R)0);
+    st.sg[s] = (R)1;
+    if (s < nst) {
+      const int d = P >> (s + 1);
+      const bool upper = (t & d) != 0;
+      T w = w96<R>(((t & (d - 1)) * (96 / (2 * d))) % 96);
+      if (inv) w.y = -w.y;
+      if (upper) { st.we[s] = w; st.sg[s] = (R)-1; }
+    }
+  }
+  st.n = nst;
+}
+
+template <typename T, typename R, int Q>
+__device__ __forceinline__ void lane_dif(T* x, int P, const LaneStages<T, R>& st) {
+#pragma unroll
+  for (int s = 0; s < 5; ++s) {
+    if (s >= st.n) break;
+    const int d = P >> (s + 1);
+    const T w = st.we[s];
+    const R sg = st.sg[s];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const T v = x[q];
+      T a;
+      a.x = __shfl_xor_sync(0xffffffffu, v.x, d);
+      a.y = __shfl_xor_sync(0xffffffffu, v.y, d);
+      x[q] = cmul(cfma_s(sg, v, a), w);
+    }
+  }
+}
+
+__device__ __forceinline__ int bitrev(int t, int P) {
+  return P <= 1 ? 0 : (int)(__brev((unsigned)t) >> (32 - __ffs(P) + 1));
+}
+
+// padded shared-memory index: one gap every 32 elements
+__device__ __forceinline__ int pidx(int s) { return s + (s >> 5); }
 
 template <typename R> __device__ __forceinline__ const cx<R>* twd(const Geom& g);
 template <> __device__ __forceinline__ const float2* twd<float>(const Geom& g) { return g.twd_f; }
@@ -606,12 +691,6 @@ int padded_len_host(int len) { return padded_len(len); }
 size_t time_smem_bytes(const Geom& g, int p) {
   // general zeta: two complex lines per spatial column
   return (size_t)(g.zeta_pi ? 1 : 2) * g.time_cpb[p] * padded_len(g.n) * (p ? sizeof(float2) : sizeof(double2));
-}
-
-cudaError_t pipe_upload_constants();
-cudaError_t upload_constants() {
-  const cudaError_t e = upload_w96();
-  return e != cudaSuccess ? e : pipe_upload_constants();
 }
 
 template <typename R, int Q>

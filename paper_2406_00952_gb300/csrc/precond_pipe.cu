@@ -1286,8 +1286,6 @@ int pipe_time_cols(int n, int zeta_pi) {
 // lines per tile of the pipelined DST passes
 int pipe_dst_lines(int L) { return kThreads / (2 * L / 32); }
 
-cudaError_t pipe_upload_constants() { return upload_w96(); }
-
 // DST pass `stage` of the FP32 apply; B.pipe_pd is the P shared by the instances it covers.
 cudaError_t pipe_dst_pass(const Batch& B, int stage, int in_slot, int out_slot) {
   const bool tm = B.pipe_pd & 64;
