@@ -553,13 +553,13 @@ cudaError_t launch_minres_wx2(const Batch& B, int sy0, int sy1, int sw, int sw2,
   k_minres_wx2<<<B.tot_vec, 256, 0, B.stream>>>(B.G, B.S, B.Sc, B.off_vec, B.count, B.active, sy0, sy1, sw, sw2, sx);
   return cudaGetLastError();
 }
-// Arnoldi index j >= 0: the kernel of exactly j + 1 vectors.  j < 0 (per-instance indices, at most jmax when
-// jmax >= 0): the smallest bound that covers them.
+// Arnoldi index j >= 0 (at most PCB_MAX_RESTART - 1): the kernel of exactly j + 1 vectors.  j < 0 (per-instance
+// indices, at most jmax when jmax >= 0): the smallest bound that covers them.
 #define PCB_EXACT(X)                                                                                      \
   X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12) X(13) X(14) X(15) X(16) X(17) X(18)     \
-  X(19) X(20) X(21) X(22) X(23) X(24) X(25) X(26) X(27) X(28) X(29) X(30) X(31) X(32) X(33)
-#define PCB_BOUNDS(X) X(2) X(4) X(6) X(8) X(10) X(12) X(14) X(16) X(20) X(24) X(33)
-static_assert(PCB_MAX_RESTART + 1 == 33, "the lists above end at the largest basis");
+  X(19) X(20) X(21) X(22) X(23) X(24) X(25) X(26) X(27) X(28) X(29) X(30) X(31) X(32)
+#define PCB_BOUNDS(X) X(2) X(4) X(6) X(8) X(10) X(12) X(14) X(16) X(20) X(24) X(32)
+static_assert(PCB_MAX_RESTART == 32, "the lists above cover the largest basis");
 cudaError_t launch_multidot(const Batch& B, int svbase, int j, int sw, int jmax) {
 #define PCB_ARGS B.G, B.S, B.Sc, B.off_vec, B.count, B.active, svbase, j, sw, B.partial, B.tot_vec
   if (j >= 0) {
@@ -571,7 +571,7 @@ cudaError_t launch_multidot(const Batch& B, int svbase, int j, int sw, int jmax)
     }
     return cudaGetLastError();
   }
-  const int need = jmax < 0 ? PCB_MAX_RESTART + 1 : jmax + 1;
+  const int need = jmax < 0 ? PCB_MAX_RESTART : jmax + 1;
 #define PCB_CASE(JB) \
   if (need <= JB) { k_multidot<JB, false><<<B.tot_vec, 256, 0, B.stream>>>(PCB_ARGS); return cudaGetLastError(); }
   PCB_BOUNDS(PCB_CASE)
@@ -581,7 +581,7 @@ cudaError_t launch_multidot(const Batch& B, int svbase, int j, int sw, int jmax)
 }
 // jmax: as for launch_multidot
 cudaError_t launch_reduce_multi(const Batch& B, int j, int pass, int jmax) {
-  const int rows = j >= 0 ? j + 1 : jmax >= 0 ? jmax + 1 : PCB_MAX_RESTART + 1;
+  const int rows = j >= 0 ? j + 1 : jmax >= 0 ? jmax + 1 : PCB_MAX_RESTART;
   k_reduce_multi<<<dim3(B.count, rows), 256, 0, B.stream>>>(B.off_vec, B.count, B.active, B.partial, B.tot_vec, j, pass,
                                                            B.Sc);
   return cudaGetLastError();
@@ -601,7 +601,7 @@ cudaError_t launch_multiaxpy(const Batch& B, int svbase, int j, int sw, int pass
     }
     return cudaGetLastError();
   }
-  const int need = jmax < 0 ? PCB_MAX_RESTART + 1 : jmax + 1;
+  const int need = jmax < 0 ? PCB_MAX_RESTART : jmax + 1;
 #define PCB_CASE(JB) \
   if (need <= JB) { k_multiaxpy<JB, false><<<B.tot_vec, 256, 0, B.stream>>>(PCB_ARGS); return cudaGetLastError(); }
   PCB_BOUNDS(PCB_CASE)
