@@ -115,13 +115,15 @@ void matvec_shape(Geom& g) {
   } else {
     g.mv_tchunk = g.n;
     // march_block: parts of the time range while that leaves at least four steps each and the columns give
-    // the device fewer than about 200 threads a multiprocessor.  The first sweep costs one or two operations
-    // a value and a read of the half; more threads than that no longer pay for it.  n = 128, theta = 1/2
-    // and 0.7, us with 1, 2, 4, 8 parts: N = 63 73, 46, 35, 35 and 76, 52, 41, 42 (4 taken); N = 95 73, 56,
-    // 56, 57 and 77, 68, 69, 72 (2); N = 127 87, 99, 87, 89 and 95, 124, 111, 115 (1); N = 191 167, 204,
-    // 183, 183 and 184, 239, 238, 240 (1).
+    // the device fewer than about 475 threads a multiprocessor: N = 127 and less.  The first sweep costs one
+    // or two operations a value and a read of the half, and pays where the marching waits for memory, which
+    // it does in a solve (its vectors come from HBM; six GMRES steps at N = 127, n = 512 7.9 ms with 4 parts,
+    // 8.9 with 1) and past the L2 cache (a product alone at N = 127, n = 512 0.33 ms with 4, 0.41 with 1).  A
+    // product whose vectors stay in L2 has it for nothing (n = 128: 87 us with either, theta = 0.7 111 and 95).
+    // At N = 191 one part is the fastest for every n and theta (n = 128: 165 us with 1, 191 with 2, 183 with 4;
+    // theta = 0.7 183, 239, 237).
     g.mv_chunks = 1;
-    while (g.mv_chunks < 8 && g.n / (2 * g.mv_chunks) >= 4 && 2LL * g.m * g.mv_chunks < 31000) g.mv_chunks *= 2;
+    while (g.mv_chunks < 8 && g.n / (2 * g.mv_chunks) >= 4 && 2LL * g.m * g.mv_chunks < 72000) g.mv_chunks *= 2;
     const int cpb = kMvThreads / g.mv_chunks;
     g.mv_blocks = 2 * ((g.m + cpb - 1) / cpb);
   }
