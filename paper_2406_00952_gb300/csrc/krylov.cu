@@ -131,9 +131,9 @@ __global__ void __launch_bounds__(256) k_minres_wx(const Geom* __restrict__ G, c
 // The updates of two iterations k, k+1 at once (coefficients wp*: iteration k, w*: k+1):
 //   u_k     = y_k     + wpc2 u_{k-2} + wpc1 u_{k-1}   -> slot w2
 //   u_{k+1} = y_{k+1} + wc2 u_{k-1} + wc1 u_k         -> slot w;   x += wpcx u_k + wcx u_{k+1}
-// 64 B a value for both instead of 96: the update of a single iteration is bound by HBM, and its FP64
-// operations (three a value and iteration) fit under the two-iteration traffic (N = 511, n = 512: two launches
-// of 2.02 ms -> one of 3.12).
+// 64 B a value for both (five reads, three writes) instead of 96: the update of a single iteration is bound by
+// HBM.  Here the six FP64 operations a value are the bound, 0.97 of the measured 529 G/s, and the traffic
+// runs at 0.81 of HBM (N = 511, n = 512: two launches of 2.02 ms -> one of 3.12).
 __global__ void __launch_bounds__(256) k_minres_wx2(const Geom* __restrict__ G, const Slots* __restrict__ S,
                                                     const Scal* __restrict__ Sc, const int* __restrict__ off, int count,
                                                     const int* __restrict__ active, int sy0, int sy1, int sw, int sw2,
@@ -181,8 +181,10 @@ __global__ void __launch_bounds__(256) k_minres_wx2(const Geom* __restrict__ G, 
 // and vector: 63 us a vector at N = 255, n = 256, against 39 us of HBM) as long as enough loads are in
 // flight: the basis values of a step are loaded in groups of eight before they are used, and the blocks
 // per SM divide the 16 per SM of a large vector.  JB is the exact count (EXACT; a predicated-off step
-// costs its issue slot) or a bound on the per-instance count.  With one value per step and the loads left
-// to the compiler, 10, 12, 15 and 17-20 vectors ran 1.2-1.5 times above that rate (12 vectors 1.18 ms).
+// costs its issue slot) or a bound on the per-instance count: 32 Arnoldi steps without a preconditioner at
+// N = 255, n = 128 take 78.2 ms with exact counts, 84.1 with bounds 24, 28 and 32 above 20 vectors.  With one
+// value per step and the loads left to the compiler, 10, 12, 15 and 17-20 vectors ran 1.2-1.5 times above the
+// FP64 rate (12 vectors 1.18 ms).
 constexpr int kGroup = 8;
 constexpr int gs_blocks(int JB) { return JB <= 8 ? 4 : 2; }
 

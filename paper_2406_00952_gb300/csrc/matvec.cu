@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(kMvThreads) k_matvec(const Geom* __restrict__ 
   if (partial && epi_kind != EPI_PLAIN) block_reduce_store(part, partial + blockIdx.x);
 }
 
-// seven blocks an SM: the columns of a 257 x 257 grid in one wave
+// Seven blocks an SM: five, six and eight are equal or slower (N = 255, n = 256).
 __global__ void __launch_bounds__(kMvThreads, 7) k_matvec_march(const Geom* __restrict__ G, const Slots* __restrict__ S,
                                                 Scal* __restrict__ Sc, const int* __restrict__ off, int count,
                                                 const int* __restrict__ active, int op, int x_slot, int out_slot,
